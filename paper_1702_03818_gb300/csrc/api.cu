@@ -245,6 +245,7 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
     else
       use_stream2d = stream_ok;
   }
+  if (use_stream3d) use_stream3d = stream3d_supported(p);  // (else the tile pass)
   if (use_stream2d && !(tune && tune->tile_y)) ty = 64;
   {
     PassArgs probe{};
@@ -263,7 +264,7 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* base = static_cast<char*>(ws);
-  if (p.kappa_kind != FRKC2_KAPPA_POWER) {
+  if (p.kappa_kind != FRKC2_KAPPA_POWER && !use_stream3d) {  // (the 3D streaming pass reads the cells')
     if (launch_faces(p, base + L.fx, base + L.fy, base + L.fz, st) != cudaSuccess) return FRKC2_ECUDA;
   }
   void* ua = base + L.ua;
@@ -397,9 +398,10 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
       return FRKC2_ECUDA;
     return FRKC2_OK;
   }
-  if (use_stream2d) {
+  if (use_stream2d || use_stream3d) {
     // interleaved complex state between passes: W buffers at ua (with va) and ub (with vb)
-    if (launch_face_pairs(p, base + L.fx, base + L.fy, base + L.fen, st) != cudaSuccess) return FRKC2_ECUDA;
+    if (use_stream2d && launch_face_pairs(p, base + L.fx, base + L.fy, base + L.fen, st) != cudaSuccess)
+      return FRKC2_ECUDA;
     a.k = 1;
     a.hx = a.hy = 1;
     a.hz = 0;
@@ -420,8 +422,9 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
         a.cb[0] = dt * plan->a_im[l] / h2;
         a.caf[0] = float(a.ca[0]);
         a.cbf[0] = float(a.cb[0]);
-        const cudaError_t e = dfloat ? launch_pass_stream2d_df(p, a, base + L.fen, st)
-                                     : launch_pass_stream2d(p, a, base + L.fen, st);
+        const cudaError_t e = use_stream3d ? launch_pass_stream3d(p, a, st)
+                              : dfloat     ? launch_pass_stream2d_df(p, a, base + L.fen, st)
+                                           : launch_pass_stream2d(p, a, base + L.fen, st);
         if (e != cudaSuccess) return FRKC2_ECUDA;
         curU = last ? u : outW;
       }
@@ -460,9 +463,7 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
       a.out_mode = outV ? PASS_IO_PLANAR : PASS_IO_REAL;
       // passes after the first may start while the previous one drains (face conductivities,
       // written before the first pass, are read before the wait for the previous pass)
-      const cudaError_t e = use_tb ? launch_pass_tb2d(p, a, st, n > 0 || q > 0)
-                            : use_stream3d ? launch_pass_stream3d(p, a, st)
-                                           : launch_pass_generic(p, a, st);
+      const cudaError_t e = use_tb ? launch_pass_tb2d(p, a, st, n > 0 || q > 0) : launch_pass_generic(p, a, st);
       if (e != cudaSuccess) return FRKC2_ECUDA;
       curU = outU;
       curV = outV;

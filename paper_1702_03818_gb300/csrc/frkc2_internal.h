@@ -131,6 +131,9 @@ cudaError_t launch_pass_wf2d(const frkc2_problem& p, const PassArgs& a, const vo
 cudaError_t launch_small1d(const frkc2_problem& p, const frkc2_plan_s& plan, double dt, int nsteps, void* u,
                            const void* fx, unsigned* status, cudaStream_t st, int cluster, int stages_per_exchange,
                            int threads_per_cta);
+int stream3d_chunks(long long blocks, int nz, long long slots);
+bool stream3d_supported(const frkc2_problem& p);
+cudaError_t launch_pass_stream3d_f32(const frkc2_problem& p, const PassArgs& a, cudaStream_t st);
 cudaError_t launch_pass_stream3d(const frkc2_problem& p, const PassArgs& a, cudaStream_t st);
 cudaError_t launch_pass_tb2d_df(const frkc2_problem& p, const PassArgs& a, cudaStream_t st, bool overlap_previous);
 cudaError_t launch_pass_stream2d_df(const frkc2_problem& p, const PassArgs& a, const void* fen, cudaStream_t st);

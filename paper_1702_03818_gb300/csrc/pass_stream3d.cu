@@ -1,22 +1,38 @@
 // 3D single-stage pass (k = 1) streaming along z, for every conductivity kind and precision.
 //
-// A CTA is TY warps; warp w is grid row y = by (TY - 2) + w - 1 and lane l is column
-// x = bx 30 + l - 1, so the CTA covers a 32 x TY column block whose outer lanes and rows are
-// halo: it outputs the 30 x (TY - 2) interior columns.  The CTA walks up its z chunk; each
-// thread keeps its own column's W(z), W(z+1) (and for kappa(u) the conductivities of both)
-// and the flux through its down face in registers.  Per plane:
-//   - x neighbours come by warp shuffle, y neighbours through a shared plane (W, and kappa
-//     for kappa(u)), double-buffered by z parity;
-//   - each cell forms the fluxes through its east, north and up faces, F = kappa_f (W_nb - W_c);
-//     the west flux is lane - 1's east flux (shuffle), the south flux row - 1's north flux (a
-//     second shared plane), the down flux the up flux of the plane below (register):
+// A CTA is nw warps; warp w holds the RY grid rows y = by OY + w RY - 1 .. + RY - 1 and lane l is
+// column x = bx 30 + l - 1, so the CTA covers a 32 x (RY nw) column block whose outer lanes and rows
+// are halo: it outputs the 30 x OY columns inside, OY = RY nw - 2.  It walks up z; each thread keeps
+// its RY columns' W and conductivity at z and z + 1 and the flux through their down faces in
+// registers.  Per plane:
+//   - each cell forms the fluxes through its east, north and up faces, F = kappa_f (W_nb - W_c); the
+//     west flux is lane - 1's east flux (shuffle), the down flux the up flux of the plane below
+//     (register), and inside a thread's rows the south flux is the north flux of the row below:
 //     f = (F_e - F_w) + (F_n - F_s) + (F_u - F_d), every face flux formed once;
-//   - for kappa(u) = 1 + c u^p every cell's kappa(W) is evaluated once per stage (when its
-//     plane is loaded) and a face takes kappa_c + kappa_nb, the factor 1/2 folded into the
-//     stage coefficients; for FIELD / CONST the face conductivities are read from the face
-//     arrays.
-// Work per output cell-stage: the halo lanes and rows add 32 TY / (30 (TY - 2)) (1.22 for
-// TY = 16); no other redundant work, against the (T + 2)^3 / T^3 halo of a tile pass.
+//   - between warps, the y exchange runs one plane ahead: a warp publishes its first row's W and
+//     kappa of plane z + 1 and its last row's north flux of plane z (formed during plane z - 1) in
+//     the same double-buffered shared write, so one barrier a plane serves both directions;
+//   - for kappa(u) = 1 + c u^p every cell's kappa(W) is evaluated once per stage (when its plane is
+//     loaded); for FIELD / CONST the cell conductivities are read (4 or 8 bytes a cell, where the
+//     three face arrays are 12 or 24).  A face takes kappa_c + kappa_nb, the factor 1/2 folded into
+//     the stage coefficients (exact).
+// Rows that are halo, or lie outside the grid, skip the x and z fluxes and the update.
+//
+// Work split: column blocks x chunks along z; neighbouring blocks of one chunk are neighbours in the
+// launch order, so CTAs that run together read the same planes and share halo columns and lines in L2
+// (one contiguous range of (block, z) per CTA instead: FP32 256^3 104 us a pass against 94).  nw is chosen
+// per grid so that the blocks cover ny with the fewest rows, the chunk count so that the waves are full.
+//
+// What bounds it: the FP64 pipe.  FP64 kappa(u) takes about 62 FP64 instructions a computed cell (24 for
+// kappa(W), 38 for the stencil and the update), FIELD / CONST 24; computed / output cells 1.14 x the
+// columns lost at ragged edges.  A pass over 160^3: FP64 kappa(u) 959 -> 668 us, MIXED 266 -> 139 us;
+// FP64 periodic FIELD 71 x 90 x 123, a step of 8 stages: 1433 -> 582 us (single rows per warp, two
+// barriers a plane, 32-plane chunks, three face arrays before).  FP32: pass_stream3d_f32.cu.
+//
+// MIXED: double state and differences, float conductivities and fluxes.  Its conversions between
+// double and float go through the integer pipe (frkc2_math.cuh), bit for bit the hardware's, because
+// a conversion takes a slot of the FP64 pipe like an addition: 10 FP64-pipe instructions a cell
+// instead of 20 (121 x 150 x 97, kappa(u), two steps of 16 stages: 5.68 -> 1.91 ms).
 #include <algorithm>
 #include <type_traits>
 
@@ -28,19 +44,17 @@
 namespace frkc2 {
 namespace {
 
-#ifndef FRKC2_S3_TY
-#define FRKC2_S3_TY 16
-#endif
-constexpr int S3_TY = FRKC2_S3_TY;  // warps (grid rows incl. 2 halo rows) per CTA
-constexpr int S3_THREADS = 32 * S3_TY;
-constexpr int S3_OX = 30, S3_OY = S3_TY - 2;  // output columns / rows per CTA
+constexpr int S3_OX = 30;          // output columns per CTA
+constexpr int S3_CHUNK = 32;       // MIXED: see flux
+constexpr int K3_FIELD = 0;        // FIELD / CONST: real conductivity read from memory (or a constant)
+constexpr int K3_POWER = 1;        // kappa(u), general exponent
+constexpr int K3_P25 = 2;          // kappa(u), exponent 2.5
 
 template <class T> struct V2s;
 template <> struct V2s<double> { using type = double2; };
 template <> struct V2s<float> { using type = float2; };
 
 __device__ __forceinline__ bool nonfinite3(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
-__device__ __forceinline__ bool nonfinite3(float v) { return (__float_as_uint(v) & 0x7f800000u) == 0x7f800000u; }
 
 __device__ __forceinline__ int wrap3(int g, int n) {
   if (g < 0) g += n;
@@ -48,224 +62,394 @@ __device__ __forceinline__ int wrap3(int g, int n) {
   return g;
 }
 
-// P25: kappa(u) with the exponent 2.5, evaluated as w^2 sqrt(w) without the general path
-template <class S, class A, bool PERIODIC, bool POWER, bool P25>
-__global__ void __launch_bounds__(S3_THREADS) k_stream3d(const PassArgs p, int zchunk) {
+// Rows of one thread and the most warps of a CTA.  160^3, kappa(u), a pass: 16 warps FP64 668 us /
+// MIXED 139 us; FP64 with 12 warps 669 us, 8 warps (2 CTAs per SM) 703 us, 4 warps (4 CTAs) 771 us:
+// with the FP64 pipe the bound, the halo rows of smaller CTAs cost more than they hide.
+constexpr int S3_RY = 2, S3_MAXW = 16;
+
+struct S3Args {
+  int nx, ny, nz;
+  int oy;                   // output rows per CTA
+  int bxn;                  // column blocks along x
+  int chunks;               // chunks along z
+  int in_real, out_real;    // the pass reads / writes the real state instead of interleaved (U, V)
+  int check_finite;
+  const void* in;
+  void* out;
+  const void* kappa;        // FIELD: cell conductivities; nullptr: the constant kc
+  double kc, kp;
+  double ca, cb;            // dt a_l / (2 dx^2): the face factor 1/2 folded in
+  unsigned* status;
+};
+
+template <class S, class A, int KIND, bool PERIODIC>
+__global__ void __launch_bounds__(32 * S3_MAXW) k_stream3d(const S3Args p) {
+  constexpr int RY = S3_RY, MAXW = S3_MAXW;
+  constexpr bool POWER = KIND != K3_FIELD;
+  constexpr bool MIX = !std::is_same<S, A>::value;
+  using S2 = typename V2s<S>::type;
+  using A2 = typename V2s<A>::type;
+  __shared__ S2 shW[2][MAXW][32];   // first row's W of the next plane
+  __shared__ A2 shK[2][MAXW][32];   // and its conductivity
+  __shared__ A2 shF[2][MAXW][32];   // last row's north flux of this plane
   // launched with programmatic stream serialization: the next launch may start its CTAs as this
   // one's exit, and every global load below comes after the previous launch has completed
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  using S2 = typename V2s<S>::type;
-  using A2 = typename V2s<A>::type;
-  __shared__ S2 shW[2][S3_TY][32];
-  __shared__ A2 shK[2][S3_TY][POWER ? 32 : 1];
-  __shared__ A2 shF[2][S3_TY][32];
-  const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+  const int lane = threadIdx.x, w = threadIdx.y, nw = blockDim.y;
   const int nx = p.nx, ny = p.ny, nz = p.nz;
-  const int gx = blockIdx.x * S3_OX + lane - 1;
-  const int gy = blockIdx.y * S3_OY + row - 1;
-  const int z0 = blockIdx.z * zchunk, z1 = min(nz, z0 + zchunk);
-  const int xr = PERIODIC ? wrap3(gx, nx) : gx;
-  const int yr = PERIODIC ? wrap3(gy, ny) : gy;
-  const bool colin = PERIODIC || (gx >= 0 && gx < nx && gy >= 0 && gy < ny);
-  const bool out_ok = lane >= 1 && lane <= 30 && row >= 1 && row <= S3_TY - 2 && gx < nx && gy < ny && gx >= 0 &&
-                      gy >= 0;
-  const size_t plane = size_t(nx) * ny;
-  const size_t col = size_t(yr) * nx + xr;  // in-plane offset of this thread's column (if colin)
-  const int in_mode = p.in_mode, out_mode = p.out_mode;
-  const S* __restrict__ Ur = static_cast<const S*>(p.U_in);
-  const S* __restrict__ Vr = static_cast<const S*>(p.V_in);
-  S* __restrict__ Uo = static_cast<S*>(p.U_out);
-  S* __restrict__ Vo = static_cast<S*>(p.V_out);
-  const A* __restrict__ FX = static_cast<const A*>(p.fx);
-  const A* __restrict__ FY = static_cast<const A*>(p.fy);
-  const A* __restrict__ FZ = static_cast<const A*>(p.fz);
-  // kappa(u): the face factor 1/2 of (kappa_c + kappa_nb)/2 is folded into the coefficients
-  const S ca = S(POWER ? 0.5 * p.ca[0] : p.ca[0]), cb = S(POWER ? 0.5 * p.cb[0] : p.cb[0]);
+  const size_t plane = size_t(nx) * ny;  // at most 2^32 (stream3d_supported)
+  const bool in_real = p.in_real, out_real = p.out_real;
+  const S ca = S(p.ca), cb = S(p.cb);
   const A kc = A(p.kc), kp = A(p.kp);
+  const S* __restrict__ Ur = static_cast<const S*>(p.in);
+  const S2* __restrict__ Wi = static_cast<const S2*>(p.in);
+  const A* __restrict__ Kf = static_cast<const A*>(p.kappa);
 
-  auto load = [&](int z) -> S2 {
-    S2 w;
-    w.x = S(0);
-    w.y = S(0);
-    int zz = z;
-    if (PERIODIC) {
-      zz = wrap3(z, nz);
-    } else if (!colin || z < 0 || z >= nz) {
-      return w;
+  const A2 a0 = {A(0), A(0)};
+  auto kap = [&](S2 v) -> A2 {
+    A2 k = a0;
+    if constexpr (KIND == K3_P25) {
+      A vx, vy;
+      if constexpr (MIX) {
+        bool slow = false;
+        vx = narrow_fast(v.x, slow);
+        vy = narrow_fast(v.y, slow);
+        while (__any_sync(0xffffffffu, slow)) {
+          vx = narrow_hw(v.x);
+          vy = narrow_hw(v.y);
+          slow = false;
+        }
+        kappa_power25_mixed(vx, vy, kc, k.x, k.y);
+      } else {
+        kappa_power25_fast(v.x, v.y, kc, k.x, k.y);
+      }
+    } else if constexpr (KIND == K3_POWER) {
+      kappa_power<A>(A(v.x), A(v.y), kc, kp, k.x, k.y);
     }
-    const size_t g = size_t(zz) * plane + col;
-    if (!in_bounds(g < size_t(nz) * plane, p.status)) return w;
-    w.x = __ldg(Ur + g);
-    if (in_mode == PASS_IO_PLANAR) w.y = __ldg(Vr + g);
-    return w;
-  };
-  // face array sizes, for the bounds-checking build's index checks
-  const size_t nfx = size_t(nz) * ny * (nx + 1), nfy = size_t(nz) * (ny + 1) * nx, nfz = size_t(nz + 1) * ny * nx;
-  auto ldf = [&](const A* F, size_t i, size_t n) -> A { return in_bounds(i < n, p.status) ? __ldg(F + i) : A(0); };
-  auto kap = [&](S2 w) -> A2 {
-    A2 k;
-    if constexpr (P25)
-      kappa_power25<A>(A(w.x), A(w.y), kc, k.x, k.y);
-    else
-      kappa_power<A>(A(w.x), A(w.y), kc, kp, k.x, k.y);
     return k;
   };
-  // face conductivities (FIELD / CONST): east (x face x+1), north (y face y+1), up (z face z+1)
-  auto face_e = [&](int z) -> A {
-    if (PERIODIC) return ldf(FX, (size_t(wrap3(z, nz)) * ny + yr) * (nx + 1) + xr + 1, nfx);
-    if (z < 0 || z >= nz || gy < 0 || gy >= ny || gx < -1 || gx >= nx) return A(0);
-    return ldf(FX, (size_t(z) * ny + gy) * (nx + 1) + gx + 1, nfx);
+  // sum of the two conductivities of a face, and the (twice the) flux
+  auto ksum = [&](A2 a, A2 b) -> A2 {
+    A2 k = a0;
+    k.x = a.x + b.x;
+    if (POWER) k.y = a.y + b.y;
+    return k;
   };
-  auto face_n = [&](int z) -> A {
-    if (PERIODIC) return ldf(FY, (size_t(wrap3(z, nz)) * (ny + 1) + yr + 1) * nx + xr, nfy);
-    if (z < 0 || z >= nz || gx < 0 || gx >= nx || gy < -1 || gy >= ny) return A(0);
-    return ldf(FY, (size_t(z) * (ny + 1) + gy + 1) * nx + gx, nfy);
-  };
-  auto face_u = [&](int z) -> A {  // z face z+1, above cell z
-    if (PERIODIC) return ldf(FZ, (size_t(wrap3(z, nz) + 1) * ny + yr) * nx + xr, nfz);
-    if (!colin || z < -1 || z >= nz) return A(0);
-    return ldf(FZ, (size_t(z + 1) * ny + gy) * nx + gx, nfz);
-  };
-  // complex flux kappa_f * d with kappa_f real (FIELD) or complex (kappa(u))
-  auto flux = [&](A2 kf, A dr, A di) -> A2 {
+  // (Which product of the imaginary part is fused is fixed here, so that a MIXED call's bits do not
+  // depend on the compiler's choice: the x and y faces one way, the z faces the other, and the down
+  // faces of every 32nd plane as the x and y faces -- the bits of a pass over 32-plane chunks.)
+  auto flux = [&](A2 kf, A dr, A di, bool zface) -> A2 {
     A2 F;
     if (POWER) {
-      F.x = kf.x * dr - kf.y * di;
-      F.y = kf.x * di + kf.y * dr;
+      F.x = fma(kf.x, dr, -mul_rn(kf.y, di));
+      F.y = zface ? fma(kf.y, dr, mul_rn(kf.x, di)) : fma(kf.x, di, mul_rn(kf.y, dr));
     } else {
       F.x = kf.x * dr;
       F.y = kf.x * di;
     }
     return F;
   };
+  // difference of two states in the arithmetic precision
+  auto diff = [&](S2 a, S2 b, bool& slow) -> A2 {
+    A2 d;
+    if constexpr (MIX) {
+      d.x = narrow_fast(a.x - b.x, slow);
+      d.y = narrow_fast(a.y - b.y, slow);
+    } else {
+      d.x = a.x - b.x;
+      d.y = a.y - b.y;
+    }
+    return d;
+  };
+  auto diff_exact = [&](S2 a, S2 b) -> A2 {
+    A2 d;
+    d.x = narrow_hw(a.x - b.x);
+    d.y = narrow_hw(a.y - b.y);
+    return d;
+  };
+  // the flux of one face on its own (the y faces between warps, and the priming planes)
+  auto face = [&](S2 a, S2 b, A2 ka, A2 kb, bool zface) -> A2 {
+    bool slow = false;
+    A2 d = diff(a, b, slow);
+    while (MIX && __any_sync(0xffffffffu, slow)) {
+      d = diff_exact(a, b);
+      slow = false;
+    }
+    return flux(ksum(ka, kb), d.x, d.y, zface);
+  };
 
-  // prime: W(z0 - 1), W(z0), W(z0 + 1) and the flux through the down face of z0
-  S2 Wc = load(z0), Wp = load(z0 + 1);
-  A2 Kc, Kp;
-  A2 Fd;
-  {
-    const S2 Wm = load(z0 - 1);
-    A2 kf;
-    if (POWER) {
-      Kc = kap(Wc);
-      Kp = kap(Wp);
-      const A2 Km = kap(Wm);
-      kf.x = Km.x + Kc.x;
-      kf.y = Km.y + Kc.y;
-    } else {
-      kf.x = face_u(z0 - 1);
-      kf.y = A(0);
-    }
-    Fd = flux(kf, A(Wc.x - Wm.x), A(Wc.y - Wm.y));
-  }
+  int b = 0;  // exchange buffer
   bool bad = false;
-  for (int z = z0; z < z1; ++z) {
-    const int b = z & 1;
-    const S2 Wpp = load(z + 2);  // the plane after next, issued early
-    A ke = A(0), kn = A(0), ku = A(0);
-    if (!POWER) {
-      ke = face_e(z);
-      kn = face_n(z);
-      ku = face_u(z);
+  const int blk = blockIdx.x, z0 = int((long long)blockIdx.y * nz / p.chunks), z1 = int((long long)(blockIdx.y + 1) * nz / p.chunks);
+  {
+    const int gx = (blk % p.bxn) * S3_OX + lane - 1;
+    const int gy0 = (blk / p.bxn) * p.oy + w * RY - 1;
+    const bool out_x = lane >= 1 && lane <= 30 && gx < nx;
+    // per row: the in-plane offset read (wrapped, or clamped to the grid: the conductivity of a
+    // Dirichlet ghost is its interior cell's), whether the row is in the grid / an output row, and
+    // whether a neighbour needs it
+    unsigned col[RY];
+    unsigned inside = 0, act = 0, need = 0;  // bits by row; act and need are warp-uniform
+    const bool xin = PERIODIC || (gx >= 0 && gx < nx);
+    const int xr = PERIODIC ? wrap3(gx, nx) : min(max(gx, 0), nx - 1);
+#pragma unroll
+    for (int r = 0; r < RY; ++r) {
+      const int gy = gy0 + r, R = w * RY + r;
+      const int yr = PERIODIC ? wrap3(gy, ny) : min(max(gy, 0), ny - 1);
+      col[r] = unsigned(yr) * unsigned(nx) + unsigned(xr);
+      if (xin && (PERIODIC || (gy >= 0 && gy < ny))) inside |= 1u << r;
+      if (R >= 1 && R <= p.oy && gy < ny) act |= 1u << r;
+      if (gy <= ny) need |= 1u << r;
     }
-    shW[b][row][lane] = Wc;
-    if (POWER) shK[b][row][lane] = Kc;
-    __syncthreads();
-    // east neighbour by shuffle (lane 31 is a halo lane: its east values are not used)
-    S2 We;
-    We.x = __shfl_down_sync(0xffffffffu, Wc.x, 1);
-    We.y = __shfl_down_sync(0xffffffffu, Wc.y, 1);
-    const int rn = row + 1 < S3_TY ? row + 1 : row;  // the top halo row has no north cell here
-    const S2 Wn = shW[b][rn][lane];
-    A2 kfe, kfn, kfu;
-    if (POWER) {
-      A2 Ke, Kn;
-      Ke.x = __shfl_down_sync(0xffffffffu, Kc.x, 1);
-      Ke.y = __shfl_down_sync(0xffffffffu, Kc.y, 1);
-      Kn = shK[b][rn][lane];
-      kfe.x = Kc.x + Ke.x;
-      kfe.y = Kc.y + Ke.y;
-      kfn.x = Kc.x + Kn.x;
-      kfn.y = Kc.y + Kn.y;
-      kfu.x = Kc.x + Kp.x;
-      kfu.y = Kc.y + Kp.y;
-    } else {
-      kfe.x = ke;
-      kfn.x = kn;
-      kfu.x = ku;
-      kfe.y = kfn.y = kfu.y = A(0);
+    auto zrow = [&](int z) -> size_t { return size_t(PERIODIC ? wrap3(z, nz) : min(max(z, 0), nz - 1)) * plane; };
+    auto load = [&](int z, size_t zo, int r) -> S2 {
+      S2 v;
+      v.x = v.y = S(0);
+      if (!PERIODIC && (z < 0 || z >= nz)) return v;
+      if (!(inside >> r & 1) || !in_bounds(zo + col[r] < size_t(nz) * plane, p.status)) return v;
+      if (in_real)
+        v.x = __ldg(Ur + zo + col[r]);
+      else
+        v = __ldg(Wi + zo + col[r]);
+      return v;
+    };
+    auto loadk = [&](size_t zo, int r) -> A2 {  // FIELD / CONST
+      A2 k = a0;
+      k.x = kc;
+      if (Kf && in_bounds(zo + col[r] < size_t(nz) * plane, p.status)) k.x = __ldg(Kf + zo + col[r]);
+      return k;
+    };
+
+    // prime: W and kappa of z0 and z0 + 1, the fluxes through the down faces of z0, and the last
+    // row's north flux of plane z0
+    S2 Wc[RY], Wp[RY];
+    A2 Kc[RY], Kp[RY], Fd[RY], Ft;
+    {
+      const size_t zm = zrow(z0 - 1), zc = zrow(z0), zp = zrow(z0 + 1);
+#pragma unroll
+      for (int r = 0; r < RY; ++r) {
+        const S2 Wm = load(z0 - 1, zm, r);
+        Wc[r] = load(z0, zc, r);
+        Wp[r] = load(z0 + 1, zp, r);
+        A2 Km;
+        if (POWER) {
+          Km = kap(Wm);
+          Kc[r] = kap(Wc[r]);
+          Kp[r] = kap(Wp[r]);
+        } else {
+          Km = loadk(zm, r);
+          Kc[r] = loadk(zc, r);
+          Kp[r] = loadk(zp, r);
+        }
+        Fd[r] = face(Wc[r], Wm, Kc[r], Km, z0 % S3_CHUNK != 0);
+      }
+      shW[b][w][lane] = Wc[0];
+      shK[b][w][lane] = Kc[0];
+      __syncthreads();
+      const int wn = w + 1 < nw ? w + 1 : w;  // (the top halo row's north flux is not used)
+      Ft = face(shW[b][wn][lane], Wc[RY - 1], Kc[RY - 1], shK[b][wn][lane], false);
+      b ^= 1;
     }
-    const A2 Fe = flux(kfe, A(We.x - Wc.x), A(We.y - Wc.y));
-    const A2 Fn = flux(kfn, A(Wn.x - Wc.x), A(Wn.y - Wc.y));
-    const A2 Fu = flux(kfu, A(Wp.x - Wc.x), A(Wp.y - Wc.y));
-    shF[b][row][lane] = Fn;
-    __syncthreads();
-    const int rs = row > 0 ? row - 1 : row;  // the bottom halo row has no south flux here
-    const A2 Fs = shF[b][rs][lane];
-    A2 Fw;
-    Fw.x = __shfl_up_sync(0xffffffffu, Fe.x, 1);
-    Fw.y = __shfl_up_sync(0xffffffffu, Fe.y, 1);
-    const A fR = ((Fe.x - Fw.x) + (Fn.x - Fs.x)) + (Fu.x - Fd.x);
-    const A fI = ((Fe.y - Fw.y) + (Fn.y - Fs.y)) + (Fu.y - Fd.y);
-    if (out_ok && in_bounds(size_t(z) * plane + col < size_t(nz) * plane, p.status)) {
-      const size_t g = size_t(z) * plane + col;
-      const S un = Wc.x + ca * S(fR) - cb * S(fI);
-      Uo[g] = un;
-      if (out_mode == PASS_IO_PLANAR) Vo[g] = Wc.y + ca * S(fI) + cb * S(fR);
-      if (p.check_finite) bad |= nonfinite3(un);
-    }
-    Fd = Fu;
-    Wc = Wp;
-    Wp = Wpp;
-    if (POWER) {
-      Kc = Kp;
-      Kp = kap(Wpp);
+    for (int z = z0; z < z1; ++z) {
+      const bool more = z + 1 < z1;
+      S2 Wl[RY];  // the plane after next, issued early
+      A2 Kl[RY];
+      const size_t zl = zrow(z + 2);
+#pragma unroll
+      for (int r = 0; r < RY; ++r) {
+        Wl[r].x = Wl[r].y = S(0);
+        Kl[r] = a0;
+        if (more) {
+          Wl[r] = load(z + 2, zl, r);
+          if (!POWER) Kl[r] = loadk(zl, r);
+        }
+      }
+      shW[b][w][lane] = Wp[0];
+      shK[b][w][lane] = Kp[0];
+      shF[b][w][lane] = Ft;
+      __syncthreads();
+      A2 Fs = shF[b][w > 0 ? w - 1 : w][lane];  // (the bottom halo row's south flux is not used)
+      const int wn = w + 1 < nw ? w + 1 : w;
+      const S2 Wnn = shW[b][wn][lane];
+      const A2 Knn = shK[b][wn][lane];
+      b ^= 1;
+      const size_t zo = size_t(z) * plane;
+#pragma unroll
+      for (int r = 0; r < RY; ++r) {
+        A2 Fn = Ft;
+        if (r + 1 < RY) Fn = face(Wc[r + 1], Wc[r], Kc[r], Kc[r + 1], false);
+        if (act >> r & 1) {
+          S2 We;
+          A2 Ke = a0;
+          We.x = __shfl_down_sync(0xffffffffu, Wc[r].x, 1);
+          We.y = __shfl_down_sync(0xffffffffu, Wc[r].y, 1);
+          Ke.x = __shfl_down_sync(0xffffffffu, Kc[r].x, 1);
+          if (POWER) Ke.y = __shfl_down_sync(0xffffffffu, Kc[r].y, 1);
+          bool slow = false;
+          A2 dE = diff(We, Wc[r], slow), dU = diff(Wp[r], Wc[r], slow);
+          while (MIX && __any_sync(0xffffffffu, slow)) {
+            dE = diff_exact(We, Wc[r]);
+            dU = diff_exact(Wp[r], Wc[r]);
+            slow = false;
+          }
+          const A2 Fe = flux(ksum(Kc[r], Ke), dE.x, dE.y, false);
+          const A2 Fu = flux(ksum(Kc[r], Kp[r]), dU.x, dU.y, true);
+          A2 Fw;
+          Fw.x = __shfl_up_sync(0xffffffffu, Fe.x, 1);
+          Fw.y = __shfl_up_sync(0xffffffffu, Fe.y, 1);
+          const A fR = ((Fe.x - Fw.x) + (Fn.x - Fs.x)) + (Fu.x - Fd[r].x);
+          const A fI = ((Fe.y - Fw.y) + (Fn.y - Fs.y)) + (Fu.y - Fd[r].y);
+          Fd[r] = Fu;
+          if (MIX && POWER && (z + 1) % S3_CHUNK == 0) Fd[r] = flux(ksum(Kc[r], Kp[r]), dU.x, dU.y, false);
+          S sR, sI;
+          if constexpr (MIX) {
+            bool sl = false;
+            sR = widen_fast(fR, sl);
+            sI = widen_fast(fI, sl);
+            while (__any_sync(0xffffffffu, sl)) {
+              sR = widen_hw(fR);
+              sI = widen_hw(fI);
+              sl = false;
+            }
+          } else {
+            sR = fR;
+            sI = fI;
+          }
+          if (out_x && in_bounds(zo + col[r] < size_t(nz) * plane, p.status)) {
+            const S un = Wc[r].x + ca * sR - cb * sI;
+            if (out_real) {
+              static_cast<S*>(p.out)[zo + col[r]] = un;
+            } else {
+              S2 o;
+              o.x = un;
+              o.y = Wc[r].y + ca * sI + cb * sR;
+              static_cast<S2*>(p.out)[zo + col[r]] = o;
+            }
+            if (p.check_finite) bad |= nonfinite3(un);
+          }
+        }
+        Fs = Fn;
+      }
+      if (more) {
+        Ft = face(Wnn, Wp[RY - 1], Kp[RY - 1], Knn, false);
+#pragma unroll
+        for (int r = 0; r < RY; ++r) {
+          Wc[r] = Wp[r];
+          Kc[r] = Kp[r];
+          Wp[r] = Wl[r];
+          if (!POWER)
+            Kp[r] = Kl[r];
+          else if (need >> r & 1)
+            Kp[r] = kap(Wl[r]);
+        }
+      }
     }
   }
   if (bad) atomicOr(p.status, ST_NONFINITE);
 }
 
-template <class S, class A, bool PERIODIC, bool POWER>
-cudaError_t launch_t(const PassArgs& a, cudaStream_t st) {
-  // z chunks of 32 planes: (32 + 2) / 32 planes loaded per plane output
-  const int zchunk = 32;
-  dim3 grid((a.nx + S3_OX - 1) / S3_OX, (a.ny + S3_OY - 1) / S3_OY, (a.nz + zchunk - 1) / zchunk);
-  // (MIXED measured 8 % slower with the specialisation, so it keeps the general evaluation)
-  const auto kern = POWER && a.kp == 2.5 && std::is_same<S, A>::value ? k_stream3d<S, A, PERIODIC, POWER, true>
-                                                                        : k_stream3d<S, A, PERIODIC, POWER, false>;
-  {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(S3_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, a, zchunk);
-    if (le != cudaSuccess) return le;
+template <class S, class A, int KIND, bool PERIODIC>
+cudaError_t launch_t(S3Args a, cudaStream_t st) {
+  constexpr int RY = S3_RY, MAXW = S3_MAXW;
+  const auto kern = k_stream3d<S, A, KIND, PERIODIC>;
+  struct Res {
+    cudaError_t err;
+    int sms, per_sm[S3_MAXW + 1];
+  };
+  static const Res res = [kern] {
+    Res r{};
+    for (int n = 1; n <= MAXW; ++n) {
+      const Residency q = query_residency(kern, 32 * n, 0);
+      if (q.err != cudaSuccess) r.err = q.err;
+      r.sms = q.sms;
+      r.per_sm[n] = q.per_sm;
+    }
+    return r;
+  }();
+  if (res.err != cudaSuccess) return res.err;
+  // warps per CTA: at least half of the most (fewer leave too few rows between the halo rows), the
+  // count that covers ny with the fewest rows, the larger of equal ones
+  int nw = 0;
+  long long best = 0;
+  for (int n = MAXW; n >= MAXW / 2; --n) {
+    const int oy = RY * n - 2;
+    const long long rows = (long long)((a.ny + oy - 1) / oy) * RY * n;
+    if (nw == 0 || rows < best) {
+      nw = n;
+      best = rows;
+    }
   }
+  a.oy = RY * nw - 2;
+  a.bxn = (a.nx + S3_OX - 1) / S3_OX;
+  const long long blocks = (long long)a.bxn * ((a.ny + a.oy - 1) / a.oy);
+  a.chunks = stream3d_chunks(blocks, a.nz, (long long)res.sms * res.per_sm[nw]);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(blocks), a.chunks, 1);
+  cfg.blockDim = dim3(32, nw, 1);
+  cfg.dynamicSmemBytes = 0;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, a);
   count_launch();
-  return cudaGetLastError();
+  return le != cudaSuccess ? le : cudaGetLastError();
 }
 
 template <class S, class A>
-cudaError_t launch_s(const frkc2_problem& p, const PassArgs& a, cudaStream_t st) {
-  const bool per = p.bc == FRKC2_BC_PERIODIC, pw = p.kappa_kind == FRKC2_KAPPA_POWER;
-  if (per) return pw ? launch_t<S, A, true, true>(a, st) : launch_t<S, A, true, false>(a, st);
-  return pw ? launch_t<S, A, false, true>(a, st) : launch_t<S, A, false, false>(a, st);
+cudaError_t launch_s(const frkc2_problem& p, const S3Args& a, cudaStream_t st) {
+  const bool per = p.bc == FRKC2_BC_PERIODIC;
+  if (p.kappa_kind != FRKC2_KAPPA_POWER) return per ? launch_t<S, A, K3_FIELD, true>(a, st) : launch_t<S, A, K3_FIELD, false>(a, st);
+  if (a.kp == 2.5) return per ? launch_t<S, A, K3_P25, true>(a, st) : launch_t<S, A, K3_P25, false>(a, st);
+  return per ? launch_t<S, A, K3_POWER, true>(a, st) : launch_t<S, A, K3_POWER, false>(a, st);
 }
 
 }  // namespace
 
+// Chunks along z: the count whose waves of CTAs (slots resident at once) take the fewest planes, two
+// more per chunk for its priming.  Column blocks of one chunk are neighbours in the launch order, so
+// the CTAs that run together read the same planes and share their halo columns and lines in L2.
+int stream3d_chunks(long long blocks, int nz, long long slots) {
+  int best = 1;
+  long long least = 0;
+  for (int c = 1; c <= std::min(nz, 256); ++c) {
+    const long long planes = (blocks * c + slots - 1) / slots * ((nz + c - 1) / c + 2);
+    if (c == 1 || planes < least) {
+      best = c;
+      least = planes;
+    }
+  }
+  return best;
+}
+
+// In-plane offsets are 32-bit, in FP32 in bytes (a larger plane takes the tile pass).
+bool stream3d_supported(const frkc2_problem& p) {
+  return p.ndim == 3 && p.n[0] * p.n[1] <= (int64_t(1) << (p.precision == FRKC2_FP32 ? 29 : 32));
+}
+
 cudaError_t launch_pass_stream3d(const frkc2_problem& p, const PassArgs& a, cudaStream_t st) {
+  S3Args s{};
+  s.nx = a.nx;
+  s.ny = a.ny;
+  s.nz = a.nz;
+  s.in_real = a.in_mode == PASS_IO_REAL;
+  s.out_real = a.out_mode == PASS_IO_REAL;
+  s.check_finite = a.check_finite;
+  s.in = a.U_in;
+  s.out = a.U_out;
+  s.kappa = p.kappa_kind == FRKC2_KAPPA_FIELD ? p.kappa : nullptr;
+  s.kc = a.kc;
+  s.kp = a.kp;
+  s.ca = 0.5 * a.ca[0];
+  s.cb = 0.5 * a.cb[0];
+  s.status = a.status;
   switch (p.precision) {
-    case FRKC2_FP64: return launch_s<double, double>(p, a, st);
-    case FRKC2_FP32: return launch_s<float, float>(p, a, st);
-    default: return launch_s<double, float>(p, a, st);
+    case FRKC2_FP64: return launch_s<double, double>(p, s, st);
+    case FRKC2_FP32: return launch_pass_stream3d_f32(p, a, st);
+    default: return launch_s<double, float>(p, s, st);
   }
 }
 
