@@ -25,10 +25,12 @@
 // pairs, chunk-major, are cut into one contiguous range per warp, so every SM gets the same
 // number of cell updates.  A range that crosses into the next chunk restarts the stream.
 #include <algorithm>
+#include <type_traits>
 
 #include <cuda_runtime.h>
 
 #include "frkc2_internal.h"
+#include "frkc2_math.cuh"
 
 namespace frkc2 {
 namespace {
@@ -63,6 +65,11 @@ __global__ void __launch_bounds__(ST_THREADS, ST_MIN_BLOCKS)
                long long nwarps_grid) {
   using S2 = typename Vec2<S>::type;
   using A2 = typename Vec2<A>::type;
+  // MIXED converts between double and float on the integer pipe (frkc2_math.cuh): a hardware conversion
+  // takes an FP64-pipe slot, 6 of the 14 of a cell-stage.  2048^2, s = 64, a step: 7704 -> 4491 us, the same
+  // bits.  Dirichlet grids keep the hardware conversions: with the others the compiler fuses other
+  // products of the face sum there, which changes the rounding of a MIXED run (8e-7 after 128 stages).
+  constexpr bool INT_CVT = !std::is_same<S, A>::value && PERIODIC;
   const int lane = threadIdx.x & 31;
   const long long gw = (long long)blockIdx.x * ST_WARPS + (threadIdx.x >> 5);
   const int nx = p.nx, ny = p.ny;
@@ -195,8 +202,27 @@ __global__ void __launch_bounds__(ST_THREADS, ST_MIN_BLOCKS)
       }
 #endif
       // differences toward the east and north neighbours
-      const A dEU = A(Ue - Wc.x), dEV = A(Ve - Wc.y);
-      const A dNU = A(Wn.x - Wc.x), dNV = A(Wn.y - Wc.y);
+      A dEU, dEV, dNU, dNV;
+      if constexpr (!INT_CVT) {
+        dEU = A(Ue - Wc.x);
+        dEV = A(Ve - Wc.y);
+        dNU = A(Wn.x - Wc.x);
+        dNV = A(Wn.y - Wc.y);
+      } else {
+        const S eU = Ue - Wc.x, eV = Ve - Wc.y, nU = Wn.x - Wc.x, nV = Wn.y - Wc.y;
+        bool slow = false;
+        dEU = narrow_fast(eU, slow);
+        dEV = narrow_fast(eV, slow);
+        dNU = narrow_fast(nU, slow);
+        dNV = narrow_fast(nV, slow);
+        while (__any_sync(0xffffffffu, slow)) {
+          dEU = narrow_hw(eU);
+          dEV = narrow_hw(eV);
+          dNU = narrow_hw(nU);
+          dNV = narrow_hw(nV);
+          slow = false;
+        }
+      }
       // west face: the west neighbour's east difference and conductivity; south face: the
       // north difference and conductivity of the row below
       const A dWU = __shfl_up_sync(0xffffffffu, dEU, 1);
@@ -204,8 +230,22 @@ __global__ void __launch_bounds__(ST_THREADS, ST_MIN_BLOCKS)
       const A kw = __shfl_up_sync(0xffffffffu, f.x, 1);
       const A fU = f.y * dNU - ks * dSU - kw * dWU + f.x * dEU;
       const A fV = f.y * dNV - ks * dSV - kw * dWV + f.x * dEV;
-      const S un = Wc.x + ca * S(fU) - cb * S(fV);
-      const S vn = Wc.y + ca * S(fV) + cb * S(fU);
+      S sU, sV;
+      if constexpr (!INT_CVT) {
+        sU = S(fU);
+        sV = S(fV);
+      } else {
+        bool slow = false;
+        sU = widen_fast(fU, slow);
+        sV = widen_fast(fV, slow);
+        while (__any_sync(0xffffffffu, slow)) {
+          sU = widen_hw(fU);
+          sV = widen_hw(fV);
+          slow = false;
+        }
+      }
+      const S un = Wc.x + ca * sU - cb * sV;
+      const S vn = Wc.y + ca * sV + cb * sU;
       if (out_ok && in_bounds(size_t(y) * nx + x < size_t(nx) * ny, p.status)) {
         const size_t g = size_t(y) * nx + x;
         if (out_mode == PASS_IO_COMPLEX) {
@@ -218,7 +258,7 @@ __global__ void __launch_bounds__(ST_THREADS, ST_MIN_BLOCKS)
           if (out_mode == PASS_IO_PLANAR) Vo[g] = vn;
         }
         if (p.check_finite) bad |= nonfinite_bits(un);
-        if (HAT) static_cast<S*>(p.H_out)[g] = __ldg(static_cast<const S*>(p.H_in) + g) + ca * S(fU);
+        if (HAT) static_cast<S*>(p.H_out)[g] = __ldg(static_cast<const S*>(p.H_in) + g) + ca * sU;
       }
       dSU = dNU;
       dSV = dNV;
