@@ -411,7 +411,8 @@ frkc2_status frkc2_bruss_rho_bound(const frkc2_bruss_problem* prob, const void* 
 
 /* Advances (v, w) by nsteps FRKC2 steps of size dt (in place; v and w distinct device arrays
  * of the problem's precision).  rho > 0: dt*rho <= beta is checked (FRKC2_EUNSTABLE).
- * tune->kernel: 0 or 1 = one persistent cooperative launch for every stage of every step,
+ * tune->kernel: 0 = library choice (FP32: passes of up to 8 stages in registers, the same
+ * results; FP64: as 1); 1 = one persistent cooperative launch for every stage of every step,
  * each CTA waiting between stages for the CTAs whose cells its stencil reads (per-CTA stage
  * flags), or for FP64 stages of more than 2048 cells a CTA at a device-wide barrier (a plan of
  * more than 1024 stages takes one launch per 1024 stages of each step); 2 = one launch per
@@ -419,7 +420,8 @@ frkc2_status frkc2_bruss_rho_bound(const frkc2_bruss_problem* prob, const void* 
  * is latched in the workspace and the launch returns early (the state is then unspecified).
  * tune->fault_inject = 1 (testing only, persistent form) makes the first wait between stages
  * wait for a count that nothing reaches.  A non-finite value in a step's output latches FRKC2_ENONFINITE.
- * Memory: 4 state reads and writes per cell-stage (32 bytes in FP32, 64 in FP64).          */
+ * Memory: 4 state reads and writes per cell-stage (32 bytes in FP32, 64 in FP64), per cell and
+ * pass in the FP32 default.                                                                */
 frkc2_status frkc2_bruss_step(frkc2_plan_t plan, const frkc2_bruss_problem* prob, double dt,
                               int nsteps, double rho, void* v, void* w, void* ws,
                               size_t ws_bytes, const frkc2_tuning* tune, void* stream);

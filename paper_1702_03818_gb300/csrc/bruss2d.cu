@@ -9,8 +9,8 @@
 // Re w, Im w), ping-ponged between two copies; the first stage of a step reads the caller's
 // real (v, w) and the last stage writes the real parts back there.
 //
-// Two launch forms:
-//  * persistent (default): ONE cooperative launch runs every stage of every step; the CTAs
+// Launch forms (FP32's default is a third one, k stages per pass in registers: bruss_tb2d.cu):
+//  * persistent (the FP64 default): ONE cooperative launch runs every stage of every step; the CTAs
 //    are all co-resident (a multiple of the SM count).  Between stages a CTA waits only for
 //    the CTAs whose cells its stencil reads (the owners of the cells within one grid row of
 //    its own range, a handful), which are also the CTAs that read its cells: each CTA
@@ -537,6 +537,21 @@ frkc2_status frkc2_bruss_step(frkc2_plan_t plan, const frkc2_bruss_problem* prob
   if (nsteps == 0) return FRKC2_OK;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* wsb = static_cast<char*>(ws);
+  if (prob->precision == FRKC2_FP32 && kern == 0 && !fault) {
+    // FP32: the temporally blocked passes at every size (200^2, s = 16, 42 steps 1859 -> 450 us against the
+    // persistent launch, 2048^2, s = 16, 10 steps 6165 -> 2218 us).  In FP64 the recomputed halo costs more
+    // than the passes save.
+    const BrussTb k = bruss_tb2d_shape(int(prob->nx), int(prob->ny), plan->s);
+    if (k.k > 0) {
+      const BrLayout L = br_layout(*prob);
+      void* P[2][4];
+      for (int b = 0; b < 2; ++b)
+        for (int c = 0; c < 4; ++c) P[b][c] = wsb + L.planes[b][c];
+      const cudaError_t te = launch_bruss_tb2d(*prob, *plan, dt, nsteps, k, static_cast<float*>(v), static_cast<float*>(w), P,
+                                               reinterpret_cast<unsigned*>(wsb + L.status), st);
+      return te == cudaSuccess ? FRKC2_OK : FRKC2_ECUDA;
+    }
+  }
   const bool per = prob->bc == FRKC2_BC_PERIODIC;
   cudaError_t e;
   if (prob->precision == FRKC2_FP64)

@@ -1,6 +1,7 @@
 // Internal declarations shared by the FRKC2 host code and kernels (not part of the C ABI).
 #pragma once
 
+#include <algorithm>
 #include <cstddef>
 #include <cstdint>
 #include <vector>
@@ -179,6 +180,29 @@ cudaError_t launch_tape_tb2d(const frkc2_problem& p, int k, const AdjTbPass& t, 
                              unsigned* status, cudaStream_t st);
 cudaError_t launch_adjrev_tb2d(const frkc2_problem& p, int k, const AdjTbPass& t, const void* fx, const void* fy,
                                unsigned* status, cudaStream_t st);
+
+// Dynamic shared memory that spreads a launch of `ctas` CTAs over the SMs: where they fit in one wave, as
+// much as leaves room for just ceil(ctas / sms) of them per SM.  CTAs of a dependent launch that starts
+// early (programmatic stream serialization) are otherwise packed onto the SMs that empty first: a pass of
+// 144 CTAs of the FP32 Brusselator on 152 SMs took 9.5 us, and 4.3 us with one CTA per SM.  The kernel's
+// MaxDynamicSharedMemorySize must be SPREAD_SMEM.
+constexpr int SPREAD_SMEM = 226 * 1024;
+inline size_t spread_smem(size_t need, long long ctas, int sms, int per_sm) {
+  const long long want = (ctas + sms - 1) / sms;  // CTAs per SM
+  if (want >= per_sm) return need;
+  const size_t room = size_t(SPREAD_SMEM) / size_t(want);  // want CTAs fit (each with its 1 KB), want + 1 do not
+  return std::max(need, want == 1 ? room : (room - 1024) / 1024 * 1024);
+}
+
+// Temporally blocked Brusselator (FP32, bruss_tb2d.cu): the shape for a grid and plan (k = 0: not
+// available), and the steps.
+struct BrussTb {
+  int cells;  // cells of a thread along each axis: 2 or 4 (regions of 32 x 32 or 64 x 64)
+  int k;      // most stages per pass
+};
+BrussTb bruss_tb2d_shape(int nx, int ny, int s);
+cudaError_t launch_bruss_tb2d(const frkc2_bruss_problem& p, const frkc2_plan_s& plan, double dt, int nsteps, BrussTb shape,
+                              float* v, float* w, void* const P[2][4], unsigned* status, cudaStream_t st);
 
 void count_launch(int n = 1);
 
