@@ -216,25 +216,23 @@ __global__ void __launch_bounds__(AS_THREADS, adj_min_blocks<S>())
 template <class S, class A, bool PERIODIC>
 cudaError_t launch_t(const AdjStreamArgs& a, cudaStream_t st) {
   const auto kern = k_adj_stream2d<S, A, PERIODIC>;
-  static const Residency res = query_residency(kern, AS_THREADS, 0);
+  static const Residency res = spread_residency(kern, AS_THREADS, 0, 0);
   if (res.err != cudaSuccess) return res.err;
   const int ncolw = (a.nx + AS_COLS - 1) / AS_COLS;
   const long long total = (long long)ncolw * a.ny;
-  long long grid = (long long)res.sms * res.per_sm;
-  const long long max_useful = (total + AS_WARPS - 1) / AS_WARPS;
-  if (grid > max_useful) grid = max_useful;
+  const SpreadGrid g = spread_grid((total + AS_WARPS - 1) / AS_WARPS, res.sms, res.per_sm);
   {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(grid), 1, 1);
+    cfg.gridDim = dim3(g.grid, 1, 1);
     cfg.blockDim = dim3(AS_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = g.smem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, a, total, grid * AS_WARPS);
+    const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, a, total, (long long)g.grid * AS_WARPS);
     if (le != cudaSuccess) return le;
   }
   count_launch();

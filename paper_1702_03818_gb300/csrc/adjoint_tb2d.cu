@@ -539,17 +539,23 @@ __global__ void __launch_bounds__(RT_THREADS, 2) k_adjrev_tb2d(const AdjTbArgs a
     }
 }
 
+// Spread over the SMs (500 x 487, s = 32, forward and backward: 1072 -> 852 us), but not where a launch takes less
+// than a third of them: launches that overlap then find free SMs, and the padding costs 1 % (300 x 277).
+size_t adj_spread(size_t need, dim3 grid, const Residency& res) {
+  const long long regions = (long long)grid.x * grid.y;
+  return 3 * regions > res.sms ? spread_smem(need, regions, res.sms, res.per_sm) : need;
+}
+
 template <bool PERIODIC>
 cudaError_t launch_rev(const AdjTbArgs& a, dim3 grid, cudaStream_t st) {
   const auto kern = k_adjrev_tb2d<PERIODIC>;
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(RevShared)));
-  if (attr != cudaSuccess) return attr;
+  static const Residency res = spread_residency(kern, RT_THREADS, sizeof(RevShared), 0);
+  if (res.err != cudaSuccess) return res.err;
   {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(RT_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = sizeof(RevShared);
+        cfg.dynamicSmemBytes = adj_spread(sizeof(RevShared), grid, res);
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -601,11 +607,16 @@ cudaError_t launch_tape_tb2d(const frkc2_problem& p, int k, const AdjTbPass& t, 
   }
   const dim3 grid = region_grid(p, k);
   const auto tk = p.bc == FRKC2_BC_PERIODIC ? k_tape_tb2d<true> : k_tape_tb2d<false>;
+  constexpr size_t fixed = 2 * 2 * 2 * 256 * sizeof(float4);  // its static shared memory
+  static const Residency res_p = spread_residency(k_tape_tb2d<true>, RT_THREADS, 0, fixed);
+  static const Residency res_d = spread_residency(k_tape_tb2d<false>, RT_THREADS, 0, fixed);
+  const Residency& res = p.bc == FRKC2_BC_PERIODIC ? res_p : res_d;
+  if (res.err != cudaSuccess) return res.err;
   {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(RT_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = adj_spread(fixed, grid, res) - fixed;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

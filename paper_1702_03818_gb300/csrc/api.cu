@@ -194,6 +194,7 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
   const bool paired_ok = plan->paired && p.ndim == 2 && p.kappa_kind != FRKC2_KAPPA_POWER;
   bool use_stream2d = false, use_tb = false, use_paired = false, use_stream3d = false, use_small1d = false;
   bool use_tb_df = false, use_wf = false;
+  int tb_cells = 4;
   const bool dfloat = p.precision == FRKC2_DFLOAT;
   const bool wf_ok = wf2d_supported(p, k, plan->s, u);
   const bool stream3d_ok = p.ndim == 3 && k == 1;
@@ -236,14 +237,20 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
       const double regions = double((nx + T - 1) / T) * ((ny + T - 1) / T) * 64.0 * 64.0 / (double(nx) * ny);
       wf_wins = 1.08 * wf2d_recompute(nx, ny, k) < regions;
     }
-    if (wf_wins || (wf_ok && !tb_ok && k > 1))
+    if (wf_wins || (wf_ok && !tb_ok && k > 1)) {
       use_wf = true;
-    else if (tb_ok && k > 1)
+    } else if (tb_ok && k > 1) {
       use_tb = true;
-    else if (stream3d_ok)
+      if (!(tune && tune->k)) {  // the library's choice of region size and stages per pass
+        const TbShape sh = tb2d_shape(int(p.n[0]), int(p.n[1]), plan->s);
+        tb_cells = sh.cells;
+        k = sh.k;
+      }
+    } else if (stream3d_ok) {
       use_stream3d = true;
-    else
+    } else {
       use_stream2d = stream_ok;
+    }
   }
   if (use_stream3d) use_stream3d = stream3d_supported(p);  // (else the tile pass)
   if (use_stream2d && !(tune && tune->tile_y)) ty = 64;
@@ -463,7 +470,7 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
       a.out_mode = outV ? PASS_IO_PLANAR : PASS_IO_REAL;
       // passes after the first may start while the previous one drains (face conductivities,
       // written before the first pass, are read before the wait for the previous pass)
-      const cudaError_t e = use_tb ? launch_pass_tb2d(p, a, st, n > 0 || q > 0) : launch_pass_generic(p, a, st);
+      const cudaError_t e = use_tb ? launch_pass_tb2d(p, a, st, n > 0 || q > 0, tb_cells) : launch_pass_generic(p, a, st);
       if (e != cudaSuccess) return FRKC2_ECUDA;
       curU = outU;
       curV = outV;

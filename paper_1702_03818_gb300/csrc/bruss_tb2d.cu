@@ -210,13 +210,7 @@ __global__ void __launch_bounds__(BT_THREADS, C == 4 ? 2 : 4) k_bruss_tb2d(const
 
 template <int C, bool PERIODIC>
 Residency bt_residency() {
-  static const Residency res = [] {
-    const auto kern = k_bruss_tb2d<C, PERIODIC>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SPREAD_SMEM);
-    Residency r = query_residency(kern, BT_THREADS, sizeof(BrTbShared<C>));
-    if (e != cudaSuccess) r.err = e;
-    return r;
-  }();
+  static const Residency res = spread_residency(k_bruss_tb2d<C, PERIODIC>, BT_THREADS, sizeof(BrTbShared<C>), 0);
   return res;
 }
 

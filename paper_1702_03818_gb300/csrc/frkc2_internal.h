@@ -112,7 +112,15 @@ size_t face_pair_bytes(const frkc2_problem& p);
 cudaError_t launch_face_pairs(const frkc2_problem& p, const void* fx, const void* fy, void* out, cudaStream_t st);
 // overlap_previous: the launch may start while the previous launch on the stream (a pass of
 // the same kind) finishes; its CTAs read the pass input only after that launch completes.
-cudaError_t launch_pass_tb2d(const frkc2_problem& p, const PassArgs& a, cudaStream_t st, bool overlap_previous);
+// cells: a thread's cells along each axis, 4 (64 x 64 regions) or 2 (32 x 32, k < 16)
+cudaError_t launch_pass_tb2d(const frkc2_problem& p, const PassArgs& a, cudaStream_t st, bool overlap_previous,
+                             int cells = 4);
+// region size and stages per pass for a grid and a plan of s stages, with the model's us a step
+struct TbShape {
+  int cells, k;
+  double us;
+};
+TbShape tb2d_shape(int nx, int ny, int s);
 bool small1d_supported(const frkc2_problem& p, int s);
 // 2D FP32 wavefront pass (pass_wf2d.cu): CTAs of WF_NW warps stream column strips of
 // 64 WF_NW cells up the grid with up to WF_KMAX stage levels in flight; rows arrive by TMA.
@@ -181,19 +189,6 @@ cudaError_t launch_tape_tb2d(const frkc2_problem& p, int k, const AdjTbPass& t, 
 cudaError_t launch_adjrev_tb2d(const frkc2_problem& p, int k, const AdjTbPass& t, const void* fx, const void* fy,
                                unsigned* status, cudaStream_t st);
 
-// Dynamic shared memory that spreads a launch of `ctas` CTAs over the SMs: where they fit in one wave, as
-// much as leaves room for just ceil(ctas / sms) of them per SM.  CTAs of a dependent launch that starts
-// early (programmatic stream serialization) are otherwise packed onto the SMs that empty first: a pass of
-// 144 CTAs of the FP32 Brusselator on 152 SMs took 9.5 us, and 4.3 us with one CTA per SM.  The kernel's
-// MaxDynamicSharedMemorySize must be SPREAD_SMEM.
-constexpr int SPREAD_SMEM = 226 * 1024;
-inline size_t spread_smem(size_t need, long long ctas, int sms, int per_sm) {
-  const long long want = (ctas + sms - 1) / sms;  // CTAs per SM
-  if (want >= per_sm) return need;
-  const size_t room = size_t(SPREAD_SMEM) / size_t(want);  // want CTAs fit (each with its 1 KB), want + 1 do not
-  return std::max(need, want == 1 ? room : (room - 1024) / 1024 * 1024);
-}
-
 // Temporally blocked Brusselator (FP32, bruss_tb2d.cu): the shape for a grid and plan (k = 0: not
 // available), and the steps.
 struct BrussTb {
@@ -222,6 +217,39 @@ Residency query_residency(K kern, int threads, size_t smem) {
   if (r.err == cudaSuccess) r.err = cudaDeviceGetAttribute(&r.sms, cudaDevAttrMultiProcessorCount, dev);
   if (r.err == cudaSuccess) r.err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.per_sm, kern, threads, smem);
   if (r.per_sm < 1) r.per_sm = 1;
+  return r;
+}
+
+// Dynamic shared memory that spreads a launch of `ctas` CTAs over the SMs: where they fit in one wave, as
+// much as leaves room for just ceil(ctas / sms) of them per SM.  CTAs of a dependent launch that starts
+// early (programmatic stream serialization) are otherwise packed onto the SMs that empty first: a pass of
+// 144 CTAs of the FP32 Brusselator on 152 SMs took 9.5 us, and 4.3 us with one CTA per SM.  The kernel's
+// MaxDynamicSharedMemorySize must be SPREAD_SMEM.
+constexpr int SPREAD_SMEM = 226 * 1024;
+inline size_t spread_smem(size_t need, long long ctas, int sms, int per_sm) {
+  const long long want = (ctas + sms - 1) / sms;  // CTAs per SM
+  if (want >= per_sm) return need;
+  const size_t room = size_t(SPREAD_SMEM) / size_t(want);  // want CTAs fit (each with its 1 KB), want + 1 do not
+  return std::max(need, want == 1 ? room : (room - 1024) / 1024 * 1024);
+}
+
+// A launch of persistent CTAs over `work` CTAs' worth of warp rows: the same number r of CTAs on every SM,
+// r the fewest that give every warp at most one row (at most per_sm), spread as above.  (256^2 FP64, a
+// stage: 5.9 us with 288 CTAs as they fell, 4.7 with 304 spread; 100^2 4.5 -> 3.05.)
+struct SpreadGrid {
+  unsigned grid;
+  size_t smem;
+};
+inline SpreadGrid spread_grid(long long work, int sms, int per_sm) {
+  const long long r = std::max<long long>(1, std::min<long long>(per_sm, (work + sms - 1) / sms));
+  return {unsigned(r * sms), spread_smem(0, r * sms, sms, per_sm)};
+}
+// query_residency for a kernel launched with such padding: `fixed` bytes of static shared memory
+template <class K>
+Residency spread_residency(K kern, int threads, size_t smem, size_t fixed) {
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SPREAD_SMEM - fixed));
+  Residency r = query_residency(kern, threads, smem);
+  if (e != cudaSuccess) r.err = e;
   return r;
 }
 

@@ -161,25 +161,23 @@ __global__ void __launch_bounds__(PR_THREADS, FRKC2_PAIRED_MIN_BLOCKS)
 template <class S, class A, bool PERIODIC>
 cudaError_t launch_t(const PassArgs& a, const void* fen, cudaStream_t st) {
   const auto kern = k_paired2d<S, A, PERIODIC>;
-  static const Residency res = query_residency(kern, PR_THREADS, 0);
+  static const Residency res = spread_residency(kern, PR_THREADS, 0, 0);
   if (res.err != cudaSuccess) return res.err;
   const int ncolw = (a.nx + PR_COLS - 1) / PR_COLS;
   const long long total = (long long)ncolw * a.ny;
-  long long grid = (long long)res.sms * res.per_sm;
-  const long long max_useful = (total + PR_WARPS - 1) / PR_WARPS;
-  if (grid > max_useful) grid = max_useful;
+  const SpreadGrid g = spread_grid((total + PR_WARPS - 1) / PR_WARPS, res.sms, res.per_sm);
   {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(grid), 1, 1);
+    cfg.gridDim = dim3(g.grid, 1, 1);
     cfg.blockDim = dim3(PR_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = g.smem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, a, fen, total, grid * PR_WARPS);
+    const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, a, fen, total, (long long)g.grid * PR_WARPS);
     if (le != cudaSuccess) return le;
   }
   count_launch();

@@ -293,24 +293,22 @@ __global__ void k_face_pairs(const A* __restrict__ fx, const A* __restrict__ fy,
 template <class S, class A, bool PERIODIC, bool HAT>
 cudaError_t launch_t(const PassArgs& a, const void* fen, cudaStream_t st) {
   const auto kern = k_stream2d<S, A, PERIODIC, HAT>;
-  static const Residency res = query_residency(kern, ST_THREADS, 0);
+  static const Residency res = spread_residency(kern, ST_THREADS, 0, 0);
   if (res.err != cudaSuccess) return res.err;
   const int ncolw = (a.nx + ST_COLS - 1) / ST_COLS;
   const long long total = (long long)ncolw * a.ny;  // (chunk, row) pairs
-  long long grid = (long long)res.sms * res.per_sm;
-  const long long max_useful = (total + ST_WARPS - 1) / ST_WARPS;
-  if (grid > max_useful) grid = max_useful;
+  const SpreadGrid g = spread_grid((total + ST_WARPS - 1) / ST_WARPS, res.sms, res.per_sm);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned(grid), 1, 1);
+  cfg.gridDim = dim3(g.grid, 1, 1);
   cfg.blockDim = dim3(ST_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = g.smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a, fen, ncolw, total, grid * ST_WARPS);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a, fen, ncolw, total, (long long)g.grid * ST_WARPS);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
 }

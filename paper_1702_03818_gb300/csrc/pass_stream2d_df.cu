@@ -223,25 +223,23 @@ __global__ void __launch_bounds__(DF_THREADS, DF_MIN_BLOCKS)
 template <bool PERIODIC, bool IN_REAL, bool OUT_REAL>
 cudaError_t launch_t(const PassArgs& a, const void* fen, cudaStream_t st) {
   const auto kern = k_stream2d_df<PERIODIC, IN_REAL, OUT_REAL>;
-  static const Residency res = query_residency(kern, DF_THREADS, 0);
+  static const Residency res = spread_residency(kern, DF_THREADS, 0, 0);
   if (res.err != cudaSuccess) return res.err;
   const int ncolw = (a.nx + DF_COLS - 1) / DF_COLS;
   const long long total = (long long)ncolw * a.ny;
-  long long grid = (long long)res.sms * res.per_sm;
-  const long long max_useful = (total + DF_WARPS - 1) / DF_WARPS;
-  if (grid > max_useful) grid = max_useful;
+  const SpreadGrid g = spread_grid((total + DF_WARPS - 1) / DF_WARPS, res.sms, res.per_sm);
   {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(grid), 1, 1);
+    cfg.gridDim = dim3(g.grid, 1, 1);
     cfg.blockDim = dim3(DF_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = g.smem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, a, static_cast<const float2*>(fen), total, grid * DF_WARPS);
+    const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, a, static_cast<const float2*>(fen), total, (long long)g.grid * DF_WARPS);
     if (le != cudaSuccess) return le;
   }
   count_launch();

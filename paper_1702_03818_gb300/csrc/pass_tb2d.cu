@@ -1,11 +1,14 @@
 // 2D temporally blocked pass for FP32 (fixed conductivity) with the state in registers:
 // k stages of Sec. 3, Eq. 13 per HBM round trip.
 //
-// A CTA of 16 x 16 threads owns a 64 x 64 region: its output tile (64 - 2k)^2 plus a k-cell
-// halo recomputed redundantly (region-edge values go stale one cell per stage, which never
-// reaches the output tile).  Thread (tx, ty) owns the 4 x 4 cells at columns 4tx..4tx+3,
-// rows 4ty..4ty+3 and keeps, for all k stages, their complex state (32 floats) and their 40
-// face conductivities in registers.  Per stage:
+// A CTA of 16 x 16 threads owns a region of 16C x 16C cells, C = 4 or 2: its output tile
+// (16C - 2k)^2 plus a k-cell halo recomputed redundantly (region-edge values go stale one cell per
+// stage, which never reaches the output tile).  Thread (tx, ty) owns the C x C cells at columns
+// C tx, rows C ty and keeps, for all k stages, their complex state (32 floats for C = 4) and their
+// face conductivities (40) in registers.  C = 4 recomputes least and serves grids that fill the
+// chip; C = 2 gives four times the CTAs for grids that would leave SMs idle (128^2: 0.78 -> 0.34 us a
+// stage, 256^2 0.80 -> 0.51; the region size and k are chosen by tb2d_shape).  Launches of less than a
+// wave are spread evenly over the SMs (spread_smem).  Per stage:
 //   - the thread's bottom and top rows go to shared memory (double-buffered by stage parity,
 //     one barrier per stage); its south and north neighbour rows come back from the threads
 //     below and above;
@@ -23,6 +26,8 @@
 // The batched launch runs the same region computation from tb2d_region.cuh; this kernel keeps
 // its own copy because, written as that shared device function, it compiled to an 11 % slower
 // pass (4.15e11 against 4.61e11 cell-stage/s at 2048^2, k = 8) with the same registers.
+#include <algorithm>
+
 #include <cuda_runtime.h>
 
 #include "frkc2_internal.h"
@@ -30,11 +35,19 @@
 namespace frkc2 {
 namespace {
 
-constexpr int RT_R = 64;          // region edge (cells)
-constexpr int RT_THREADS = 256;   // 16 x 16 threads of 4 x 4 cells
-#ifndef FRKC2_TBR_MIN_BLOCKS
-#define FRKC2_TBR_MIN_BLOCKS 2
-#endif
+constexpr int RT_THREADS = 256;   // 16 x 16 threads of C x C cells
+
+// a row of C cells of one component, as it goes through shared memory, and as cell pairs
+template <int C> struct Row;
+template <> struct Row<4> { using type = float4; };
+template <> struct Row<2> { using type = float2; };
+__device__ __forceinline__ float4 row_of(const float2 (&a)[2]) { return make_float4(a[0].x, a[0].y, a[1].x, a[1].y); }
+__device__ __forceinline__ float2 row_of(const float2 (&a)[1]) { return a[0]; }
+__device__ __forceinline__ void row_get(float4 v, float2 (&a)[2]) {
+  a[0] = make_float2(v.x, v.y);
+  a[1] = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void row_get(float2 v, float2 (&a)[1]) { a[0] = v; }
 
 __device__ __forceinline__ int wrap_r(int g, int n) {
   if (g >= 0 && g < n) return g;
@@ -47,10 +60,12 @@ __device__ __forceinline__ int wrap_r(int g, int n) {
 // a - b on both halves in one packed instruction (sm_100 family)
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
 
-template <bool PERIODIC>
-__global__ void __launch_bounds__(RT_THREADS, FRKC2_TBR_MIN_BLOCKS) k_tb2d_reg(const PassArgs p) {
-  __shared__ float4 sh_bot[2][2][16][16];  // [stage parity][U, V][ty][tx]: the thread's row 0
-  __shared__ float4 sh_top[2][2][16][16];  // its row 3
+template <int C, bool PERIODIC>
+__global__ void __launch_bounds__(RT_THREADS, C == 4 ? 2 : 4) k_tb2d_reg(const PassArgs p) {
+  using R = typename Row<C>::type;
+  constexpr int H = C / 2, RT_R = 16 * C;  // pairs of a row; region edge (cells)
+  __shared__ R sh_bot[2][2][16][16];  // [stage parity][U, V][ty][tx]: the thread's first row
+  __shared__ R sh_top[2][2][16][16];  // its last row
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int k = p.k;
   const int T = RT_R - 2 * k;
@@ -66,11 +81,11 @@ __global__ void __launch_bounds__(RT_THREADS, FRKC2_TBR_MIN_BLOCKS) k_tb2d_reg(c
 
   // wrapped (periodic) or raw (Dirichlet) grid rows / columns of the thread's cells; the fifth
   // entry is the next row / column (north and east faces)
-  int gyr[5], gxc[5];
-  bool yin[5], xin[5];
+  int gyr[C + 1], gxc[C + 1];
+  bool yin[C + 1], xin[C + 1];
 #pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const int gx = x0 + 4 * tx + i, gy = y0 + 4 * ty + i;
+  for (int i = 0; i < C + 1; ++i) {
+    const int gx = x0 + C * tx + i, gy = y0 + C * ty + i;
     gxc[i] = PERIODIC ? wrap_r(gx, nx) : gx;
     gyr[i] = PERIODIC ? wrap_r(gy, ny) : gy;
     xin[i] = gx >= 0 && gx < nx;
@@ -78,13 +93,13 @@ __global__ void __launch_bounds__(RT_THREADS, FRKC2_TBR_MIN_BLOCKS) k_tb2d_reg(c
   }
   // fx[r][c]: x face c of row r (the west face of cell c; c = 4 is the east face of cell 3);
   // fy[r][c]: y face r of column c (the south face of row r; r = 4 is the north face of row 3)
-  float fx[4][5], fy[5][4];
+  float fx[C][C + 1], fy[C + 1][C];
   unsigned inside = 0;  // Dirichlet: bit 4r + c set if cell (r, c) lies in the grid
 #pragma unroll
-  for (int r = 0; r < 5; ++r) {
+  for (int r = 0; r < C + 1; ++r) {
 #pragma unroll
-    for (int c = 0; c < 5; ++c) {
-      if (r < 4) {
+    for (int c = 0; c < C + 1; ++c) {
+      if (r < C) {
         float v = 0.f;
         if (PERIODIC || (yin[r] && gxc[c] >= 0 && gxc[c] <= nx)) {
           const size_t fi = size_t(gyr[r]) * (nx + 1) + gxc[c];
@@ -92,14 +107,14 @@ __global__ void __launch_bounds__(RT_THREADS, FRKC2_TBR_MIN_BLOCKS) k_tb2d_reg(c
         }
         fx[r][c] = v;
       }
-      if (c < 4) {
+      if (c < C) {
         float v = 0.f;
         if (PERIODIC || (xin[c] && gyr[r] >= 0 && gyr[r] <= ny)) {
           const size_t fi = size_t(gyr[r]) * nx + gxc[c];
           if (in_bounds(fi < size_t(ny + 1) * nx, p.status)) v = FY[fi];
         }
         fy[r][c] = v;
-        if (r < 4 && xin[c] && yin[r]) inside |= 1u << (4 * r + c);
+        if (r < C && xin[c] && yin[r]) inside |= 1u << (C * r + c);
       }
     }
   }
@@ -107,17 +122,17 @@ __global__ void __launch_bounds__(RT_THREADS, FRKC2_TBR_MIN_BLOCKS) k_tb2d_reg(c
   // the previous pass's state is complete and visible after this (a no-op for a launch
   // without the programmatic-serialization attribute)
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  float2 U2[4][2], V2[4][2], FY2[5][2];
+  float2 U2[C][H], V2[C][H], FY2[C + 1][H];
 #pragma unroll
-  for (int r = 0; r < 5; ++r)
+  for (int r = 0; r < C + 1; ++r)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) FY2[r][h] = make_float2(fy[r][2 * h], fy[r][2 * h + 1]);
+    for (int h = 0; h < H; ++h) FY2[r][h] = make_float2(fy[r][2 * h], fy[r][2 * h + 1]);
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+  for (int r = 0; r < C; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
+    for (int c = 0; c < C; ++c) {
       float uu = 0.f, vv = 0.f;
-      if (PERIODIC || (inside & (1u << (4 * r + c)))) {
+      if (PERIODIC || (inside & (1u << (C * r + c)))) {
         const size_t g = size_t(gyr[r]) * nx + gxc[c];
         if (in_bounds(g < size_t(nx) * ny, p.status)) {
           uu = Uin[g];
@@ -133,50 +148,65 @@ __global__ void __launch_bounds__(RT_THREADS, FRKC2_TBR_MIN_BLOCKS) k_tb2d_reg(c
       }
     }
 
-  const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+  const float2 z2 = make_float2(0.f, 0.f);
   for (int j = 0; j < k; ++j) {
     const int b = j & 1;
-    sh_bot[b][0][ty][tx] = make_float4(U2[0][0].x, U2[0][0].y, U2[0][1].x, U2[0][1].y);
-    sh_bot[b][1][ty][tx] = make_float4(V2[0][0].x, V2[0][0].y, V2[0][1].x, V2[0][1].y);
-    sh_top[b][0][ty][tx] = make_float4(U2[3][0].x, U2[3][0].y, U2[3][1].x, U2[3][1].y);
-    sh_top[b][1][ty][tx] = make_float4(V2[3][0].x, V2[3][0].y, V2[3][1].x, V2[3][1].y);
+    sh_bot[b][0][ty][tx] = row_of(U2[0]);
+    sh_bot[b][1][ty][tx] = row_of(V2[0]);
+    sh_top[b][0][ty][tx] = row_of(U2[C - 1]);
+    sh_top[b][1][ty][tx] = row_of(V2[C - 1]);
     __syncthreads();
     // the region's outermost thread rows have no neighbour row here: their edge goes stale
-    const float4 su4 = ty > 0 ? sh_top[b][0][ty - 1][tx] : z4, sv4 = ty > 0 ? sh_top[b][1][ty - 1][tx] : z4;
-    const float4 nu4 = ty < 15 ? sh_bot[b][0][ty + 1][tx] : z4, nv4 = ty < 15 ? sh_bot[b][1][ty + 1][tx] : z4;
+    float2 su2[H], sv2[H], nu2[H], nv2[H];
+#pragma unroll
+    for (int h = 0; h < H; ++h) su2[h] = sv2[h] = nu2[h] = nv2[h] = z2;
+    if (ty > 0) {
+      row_get(sh_top[b][0][ty - 1][tx], su2);
+      row_get(sh_top[b][1][ty - 1][tx], sv2);
+    }
+    if (ty < 15) {
+      row_get(sh_bot[b][0][ty + 1][tx], nu2);
+      row_get(sh_bot[b][1][ty + 1][tx], nv2);
+    }
     const float ca = p.caf[j], cb = p.cbf[j];
     const float2 ca2 = make_float2(ca, ca), cb2 = make_float2(cb, cb), ncb2 = make_float2(-cb, -cb);
-    const float2 su2[2] = {make_float2(su4.x, su4.y), make_float2(su4.z, su4.w)};
-    const float2 sv2[2] = {make_float2(sv4.x, sv4.y), make_float2(sv4.z, sv4.w)};
-    const float2 nu2[2] = {make_float2(nu4.x, nu4.y), make_float2(nu4.z, nu4.w)};
-    const float2 nv2[2] = {make_float2(nv4.x, nv4.y), make_float2(nv4.z, nv4.w)};
     // differences across the south faces of the current row: W(r) - W(r - 1)
-    float2 dsU[2], dsV[2];
+    float2 dsU[H], dsV[H];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < H; ++h) {
       dsU[h] = sub2(U2[0][h], su2[h]);
       dsV[h] = sub2(V2[0][h], sv2[h]);
     }
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
+    for (int r = 0; r < C; ++r) {
       // columns beyond the thread's own, before this row is updated
-      const float wU = __shfl_up_sync(0xffffffffu, U2[r][1].y, 1, 16);
-      const float wV = __shfl_up_sync(0xffffffffu, V2[r][1].y, 1, 16);
+      const float wU = __shfl_up_sync(0xffffffffu, U2[r][H - 1].y, 1, 16);
+      const float wV = __shfl_up_sync(0xffffffffu, V2[r][H - 1].y, 1, 16);
       const float eU = __shfl_down_sync(0xffffffffu, U2[r][0].x, 1, 16);
       const float eV = __shfl_down_sync(0xffffffffu, V2[r][0].x, 1, 16);
-      const float u[6] = {wU, U2[r][0].x, U2[r][0].y, U2[r][1].x, U2[r][1].y, eU};
-      const float v[6] = {wV, V2[r][0].x, V2[r][0].y, V2[r][1].x, V2[r][1].y, eV};
-      // dx[c]: across x face c, W(c) - W(c - 1), each formed once for the two cells of the face
-      float dxU[5], dxV[5];
+      float u[C + 2], v[C + 2];
+      u[0] = wU;
+      v[0] = wV;
 #pragma unroll
-      for (int c = 0; c < 5; ++c) {
+      for (int h = 0; h < H; ++h) {
+        u[2 * h + 1] = U2[r][h].x;
+        u[2 * h + 2] = U2[r][h].y;
+        v[2 * h + 1] = V2[r][h].x;
+        v[2 * h + 2] = V2[r][h].y;
+      }
+      u[C + 1] = eU;
+      v[C + 1] = eV;
+      // dx[c]: across x face c, W(c) - W(c - 1), each formed once for the two cells of the face
+      float dxU[C + 1], dxV[C + 1];
+#pragma unroll
+      for (int c = 0; c < C + 1; ++c) {
         dxU[c] = u[c + 1] - u[c];
         dxV[c] = v[c + 1] - v[c];
       }
       // x part of f per cell, written straight into the halves of the pairs
-      float2 fU[2], fV[2];
+      float2 fU[H], fV[H];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
+      for (int h = 0; h < H; ++h) {
         const int c = 2 * h;
         fU[h].x = fx[r][c + 1] * dxU[c + 1] - fx[r][c] * dxU[c];
         fU[h].y = fx[r][c + 2] * dxU[c + 2] - fx[r][c + 1] * dxU[c + 1];
@@ -184,9 +214,9 @@ __global__ void __launch_bounds__(RT_THREADS, FRKC2_TBR_MIN_BLOCKS) k_tb2d_reg(c
         fV[h].y = fx[r][c + 2] * dxV[c + 2] - fx[r][c + 1] * dxV[c + 1];
       }
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float2 nU = r < 3 ? U2[r + 1][h] : nu2[h];
-        const float2 nV = r < 3 ? V2[r + 1][h] : nv2[h];
+      for (int h = 0; h < H; ++h) {
+        const float2 nU = r < C - 1 ? U2[r < C - 1 ? r + 1 : r][h] : nu2[h];
+        const float2 nV = r < C - 1 ? V2[r < C - 1 ? r + 1 : r][h] : nv2[h];
         const float2 dnU = sub2(nU, U2[r][h]), dnV = sub2(nV, V2[r][h]);
         // y part, two cells per instruction: f += k_n d_n - k_s d_s
         const float2 nks = make_float2(-FY2[r][h].x, -FY2[r][h].y);
@@ -196,8 +226,8 @@ __global__ void __launch_bounds__(RT_THREADS, FRKC2_TBR_MIN_BLOCKS) k_tb2d_reg(c
         float2 un = __ffma2_rn(ncb2, fV[h], __ffma2_rn(ca2, fU[h], U2[r][h]));
         float2 vn = __ffma2_rn(cb2, fU[h], __ffma2_rn(ca2, fV[h], V2[r][h]));
         if (!PERIODIC) {
-          if (!(inside & (1u << (4 * r + 2 * h)))) un.x = vn.x = 0.f;
-          if (!(inside & (1u << (4 * r + 2 * h + 1)))) un.y = vn.y = 0.f;
+          if (!(inside & (1u << (C * r + 2 * h)))) un.x = vn.x = 0.f;
+          if (!(inside & (1u << (C * r + 2 * h + 1)))) un.y = vn.y = 0.f;
         }
         U2[r][h] = un;
         V2[r][h] = vn;
@@ -212,13 +242,13 @@ __global__ void __launch_bounds__(RT_THREADS, FRKC2_TBR_MIN_BLOCKS) k_tb2d_reg(c
   float* __restrict__ Vo = static_cast<float*>(p.V_out);
   bool bad = false;
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int ry = 4 * ty + r;
+  for (int r = 0; r < C; ++r) {
+    const int ry = C * ty + r;
     const int gy = y0 + ry;
     if (ry < k || ry >= RT_R - k || gy >= ny) continue;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int rx = 4 * tx + c;
+    for (int c = 0; c < C; ++c) {
+      const int rx = C * tx + c;
       const int gx = x0 + rx;
       if (rx < k || rx >= RT_R - k || gx >= nx) continue;
       const size_t g = size_t(gy) * nx + gx;
@@ -232,30 +262,84 @@ __global__ void __launch_bounds__(RT_THREADS, FRKC2_TBR_MIN_BLOCKS) k_tb2d_reg(c
   if (bad) atomicOr(p.status, ST_NONFINITE);
 }
 
-}  // namespace
-
-bool tb2d_supported(const frkc2_problem& p, int k) {
-  return p.ndim == 2 && p.precision == FRKC2_FP32 && p.kappa_kind != FRKC2_KAPPA_POWER && k >= 1 &&
-         2 * k < RT_R;
+template <int C, bool PERIODIC>
+Residency tb_residency() {
+  static const Residency res =
+      spread_residency(k_tb2d_reg<C, PERIODIC>, RT_THREADS, 0, sizeof(typename Row<C>::type) * 2 * 2 * 2 * 256);
+  return res;
 }
 
-cudaError_t launch_pass_tb2d(const frkc2_problem& p, const PassArgs& a, cudaStream_t st, bool overlap_previous) {
-  (void)p;
-  const int T = RT_R - 2 * a.k;
+template <int C, bool PERIODIC>
+cudaError_t launch_c(const PassArgs& a, cudaStream_t st, bool overlap_previous) {
+  const Residency res = tb_residency<C, PERIODIC>();
+  if (res.err != cudaSuccess) return res.err;
+  const int T = 16 * C - 2 * a.k;
+  const size_t stat = sizeof(typename Row<C>::type) * 2 * 2 * 2 * 256;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((a.nx + T - 1) / T, (a.ny + T - 1) / T, 1);
   cfg.blockDim = dim3(RT_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = spread_smem(stat, (long long)cfg.gridDim.x * cfg.gridDim.y, res.sms, res.per_sm) - stat;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = overlap_previous ? 1 : 0;
-  const cudaError_t e = a.bc == FRKC2_BC_PERIODIC ? cudaLaunchKernelEx(&cfg, k_tb2d_reg<true>, a)
-                                                  : cudaLaunchKernelEx(&cfg, k_tb2d_reg<false>, a);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_tb2d_reg<C, PERIODIC>, a);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace
+
+// Time of a pass of k stages over `regions` regions in us, fitted to measurements on periodic grids of 64^2 to
+// 2048^2 (k = 2 .. 10): a wave by the CTAs an SM holds, and waves that overlap by c at their ends.
+// Model / measured: C = 2, k = 8, 128^2 3.1 / 3.0, 256^2 4.1 / 4.1; C = 4, k = 6, 1021 x 777 9.4 / 9.2, k = 7, 1024^2
+// 15.1 / 14.8, k = 8, 2048^2 61.0 / 61.1.
+static double tb2d_pass_us(int C, int k, long long regions, int sms) {
+  auto wave = [&](long long ctas) {
+    const long long r = (ctas + sms - 1) / sms;  // CTAs per SM
+    if (C == 4) return r <= 1 ? 4.6 + 0.3 * k : 5.8 + 0.6 * k;
+    return r <= 1 ? 2.0 + 0.135 * k : r == 2 ? 2.4 + 0.21 * k : r == 3 ? 2.4 + 0.38 * k : 2.0 + 0.64 * k;
+  };
+  const double c = C == 4 ? 1.6 : 0.3 * k;
+  const long long slots = (long long)(C == 4 ? 2 : 4) * sms, full = regions / slots, rest = regions % slots;
+  return double(full) * (wave(slots) - c) + (rest ? wave(rest) : c);
+}
+
+static TbShape tb2d_best(int C, int nx, int ny, int s, int kmax) {
+  static const int sms = [] {
+    int dev = 0, n = 152;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      n = 152;
+    return n;
+  }();
+  TbShape best{C, 1, 0.0};
+  for (int k = 1; k <= std::min(s, kmax); ++k) {
+    auto pass = [&](int q) {
+      const int T = 16 * C - 2 * q;
+      return tb2d_pass_us(C, q, (long long)((nx + T - 1) / T) * ((ny + T - 1) / T), sms);
+    };
+    const double us = (s / k) * pass(k) + (s % k ? pass(s % k) : 0.0);
+    if (k == 1 || us < best.us) best = TbShape{C, k, us};
+  }
+  return best;
+}
+
+TbShape tb2d_shape(int nx, int ny, int s) {
+  const TbShape a = tb2d_best(2, nx, ny, s, 10), b = tb2d_best(4, nx, ny, s, 12);
+  return a.us < b.us ? a : b;
+}
+
+bool tb2d_supported(const frkc2_problem& p, int k) {
+  return p.ndim == 2 && p.precision == FRKC2_FP32 && p.kappa_kind != FRKC2_KAPPA_POWER && k >= 1 && 2 * k < 64;
+}
+
+cudaError_t launch_pass_tb2d(const frkc2_problem& p, const PassArgs& a, cudaStream_t st, bool overlap_previous, int cells) {
+  (void)p;
+  const bool per = a.bc == FRKC2_BC_PERIODIC;
+  if (cells == 2) return per ? launch_c<2, true>(a, st, overlap_previous) : launch_c<2, false>(a, st, overlap_previous);
+  return per ? launch_c<4, true>(a, st, overlap_previous) : launch_c<4, false>(a, st, overlap_previous);
 }
 
 }  // namespace frkc2

@@ -49,14 +49,15 @@ __global__ void __launch_bounds__(RT_THREADS, 2) k_tb2d_df(const PassArgs p) {
 template <bool PERIODIC, bool IN_REAL, bool OUT_REAL>
 cudaError_t launch_t(const PassArgs& a, cudaStream_t st, bool overlap_previous) {
   const auto kern = k_tb2d_df<PERIODIC, IN_REAL, OUT_REAL>;
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(DfShared)));
-  if (attr != cudaSuccess) return attr;
+  static const Residency res = spread_residency(kern, RT_THREADS, sizeof(DfShared), 0);
+  if (res.err != cudaSuccess) return res.err;
   const int T = RT_R - 2 * a.k;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((a.nx + T - 1) / T, (a.ny + T - 1) / T, 1);
   cfg.blockDim = dim3(RT_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = sizeof(DfShared);
+  // (k stays 8 at every size: another k would run other stages in the first and last pass, whose
+  // instantiations round some fluxes differently)
+  cfg.dynamicSmemBytes = spread_smem(sizeof(DfShared), (long long)cfg.gridDim.x * cfg.gridDim.y, res.sms, res.per_sm);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
