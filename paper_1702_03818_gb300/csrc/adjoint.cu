@@ -290,8 +290,8 @@ struct AdjCtx {
   cudaStream_t st;
   size_t N, SB, slot;
   bool stream2d;  // 2D fixed conductivity: streaming kernels, interleaved tape and lambda
-  bool tb;        // ... in FP32: temporally blocked tape and reverse passes of tbk stages
-  int tbk;
+  bool tb;        // ... in FP32: temporally blocked tape and reverse passes
+  int tape_k, rev_k;  // their most stages
   int tx, ty, tz;
   char* ckpt(int j) const { return base + L.ckpt + size_t(j) * slot; }
   char* tape(int q, int l) const { return base + L.tape + (size_t(q) * s + l) * 2 * slot; }
@@ -323,8 +323,9 @@ frkc2_status adj_setup(AdjCtx& C, frkc2_plan_t plan, const frkc2_problem* prob, 
   C.SB = state_bytes(p.precision);
   C.slot = align256(C.N * C.SB);
   C.stream2d = p.ndim == 2 && p.kappa_kind != FRKC2_KAPPA_POWER;
-  C.tbk = 8;
-  C.tb = C.stream2d && adj_tb2d_supported(p, C.tbk);
+  C.tb = C.stream2d && adj_tb2d_supported(p, 8);
+  C.tape_k = C.tb ? adj_tb2d_k(p, C.s, false) : 0;
+  C.rev_k = C.tb ? adj_tb2d_k(p, C.s, true) : 0;
   default_tiles(p, 1, &C.tx, &C.ty, &C.tz);
   if (p.ndim < 2) C.ty = 1;
   if (p.ndim < 3) C.tz = 1;
@@ -360,7 +361,7 @@ bool run_segment(const AdjCtx& C, int j) {
     for (int q = 0; q < m; ++q)
       for (int l0 = 0; l0 < C.s;) {
         AdjTbPass t{};
-        t.nst = std::min(C.tbk, C.s - l0);
+        t.nst = std::min(C.tape_k, C.s - l0);
         t.in = l0 == 0 ? C.w0(j, q) : C.tape(q, l0);
         t.in_complex = l0 != 0;
         for (int jj = 0; jj < t.nst; ++jj) {
@@ -370,7 +371,7 @@ bool run_segment(const AdjCtx& C, int j) {
           t.cb[jj] = C.dt * C.plan->a_im[l] / C.h2;
         }
         t.last_real = l0 + t.nst == C.s;
-        if (launch_tape_tb2d(p, C.tbk, t, C.base + C.L.fx, C.base + C.L.fy, a.status, C.st) != cudaSuccess)
+        if (launch_tape_tb2d(p, t.nst, t, C.base + C.L.fx, C.base + C.L.fy, a.status, C.st) != cudaSuccess)
           return false;
         l0 += t.nst;
       }
@@ -428,7 +429,9 @@ bool run_segment_plain_tb(const AdjCtx& C, int j) {
   const void* curU = C.ckpt(j);
   const void* curV = nullptr;
   const int n0 = j * C.c, m = std::min(C.c, C.nsteps - n0);
-  const int k = C.tbk, npass = (C.s + k - 1) / k;
+  // (these round as the tape passes do: a segment gives the same states with and without a tape)
+  const TbShape shape = tb2d_shape_even(int(p.n[0]), int(p.n[1]), C.s);
+  const int k = shape.k, npass = (C.s + k - 1) / k;
   for (int q = 0; q < m; ++q)
     for (int ps = 0; ps < npass; ++ps) {
       const int l0 = ps * k, kq = std::min(k, C.s - l0);
@@ -451,7 +454,7 @@ bool run_segment_plain_tb(const AdjCtx& C, int j) {
       }
       a.in_mode = curV ? PASS_IO_PLANAR : PASS_IO_REAL;
       a.out_mode = outV ? PASS_IO_PLANAR : PASS_IO_REAL;
-      if (launch_pass_tb2d(p, a, C.st, q > 0 || ps > 0) != cudaSuccess) return false;
+      if (launch_pass_tb2d(p, a, C.st, q > 0 || ps > 0, shape.cells) != cudaSuccess) return false;
       curU = outU;
       curV = outV;
     }
@@ -505,10 +508,10 @@ frkc2_status adj_backward(const AdjCtx& C, const void* g, void* dJdu0, void* dJd
     if (j != C.L.nseg - 1 && !run_segment(C, j)) return FRKC2_ECUDA;
     const int m = std::min(C.c, C.nsteps - j * C.c);
     for (int q = m - 1; q >= 0; --q) {
-      if (C.tb) {  // passes of up to tbk stages, last stage first
+      if (C.tb) {  // passes of up to rev_k stages, last stage first
         for (int lhi = C.s; lhi > 0;) {
           AdjTbPass t{};
-          t.nst = std::min(C.tbk, lhi);
+          t.nst = std::min(C.rev_k, lhi);
           for (int jj = 0; jj < t.nst; ++jj) {
             const int l = lhi - 1 - jj;
             t.W[jj] = l == 0 ? C.w0(j, q) : C.tape(q, l);
@@ -525,7 +528,7 @@ frkc2_status adj_backward(const AdjCtx& C, const void* g, void* dJdu0, void* dJd
           }
           t.L_out = lam[cur ^ 1];
           t.dk = dk;
-          if (launch_adjrev_tb2d(p, C.tbk, t, C.base + C.L.fx, C.base + C.L.fy,
+          if (launch_adjrev_tb2d(p, t.nst, t, C.base + C.L.fx, C.base + C.L.fy,
                                  reinterpret_cast<unsigned*>(C.base + C.L.status), C.st) != cudaSuccess)
             return FRKC2_ECUDA;
           cur ^= 1;

@@ -143,7 +143,9 @@ __device__ __forceinline__ void set_half(float2& a, int i, float v) {
 // ------------------------------------------------------------------------------------------
 // Tape pass: forward stages, every stage state of the output tile written.
 
-template <bool PERIODIC>
+// PAIRS (nx and k even): cells 2h and 2h + 1 of a row are one aligned 16-byte access, loaded and stored as
+// such (template argument: as a run-time branch it slowed the other path by 13 %)
+template <bool PERIODIC, bool PAIRS>
 __global__ void __launch_bounds__(RT_THREADS, 2) k_tape_tb2d(const AdjTbArgs a) {
   __shared__ float4 sh_bot[2][2][16][16];  // [parity][U, V][ty][tx]: the thread's row 0
   __shared__ float4 sh_top[2][2][16][16];  // its row 3
@@ -171,24 +173,37 @@ __global__ void __launch_bounds__(RT_THREADS, 2) k_tape_tb2d(const AdjTbArgs a) 
       FY2[r][h] = make_float2(face_y<PERIODIC>(R, a.fy, nx, ny, r, 2 * h), face_y<PERIODIC>(R, a.fy, nx, ny, r, 2 * h + 1));
   }
   float2 U2[4][2], V2[4][2];
+  if (PAIRS && a.in_complex) {
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < 4; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      float uu = 0.f, vv = 0.f;
-      if (PERIODIC || (R.inside & (1u << (4 * r + c)))) {
-        const size_t g = size_t(R.gyr[r]) * nx + R.gxc[c];
-        if (a.in_complex) {
-          const float2 w = static_cast<const float2*>(a.in)[g];
-          uu = w.x;
-          vv = w.y;
-        } else {
-          uu = static_cast<const float*>(a.in)[g];
-        }
+      for (int h = 0; h < 2; ++h) {
+        float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (PERIODIC || (R.inside & (1u << (4 * r + 2 * h))))
+          w = *reinterpret_cast<const float4*>(static_cast<const float2*>(a.in) + size_t(R.gyr[r]) * nx + R.gxc[2 * h]);
+        U2[r][h] = make_float2(w.x, w.z);
+        V2[r][h] = make_float2(w.y, w.w);
       }
-      set_half(U2[r][c >> 1], c & 1, uu);
-      set_half(V2[r][c >> 1], c & 1, vv);
-    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        float uu = 0.f, vv = 0.f;
+        if (PERIODIC || (R.inside & (1u << (4 * r + c)))) {
+          const size_t g = size_t(R.gyr[r]) * nx + R.gxc[c];
+          if (a.in_complex) {
+            const float2 w = static_cast<const float2*>(a.in)[g];
+            uu = w.x;
+            vv = w.y;
+          } else {
+            uu = static_cast<const float*>(a.in)[g];
+          }
+        }
+        set_half(U2[r][c >> 1], c & 1, uu);
+        set_half(V2[r][c >> 1], c & 1, vv);
+      }
+  }
 
   bool bad = false;
   const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -256,20 +271,30 @@ __global__ void __launch_bounds__(RT_THREADS, 2) k_tape_tb2d(const AdjTbArgs a) 
     // this stage's state of the output tile to the tape
     const bool real_out = a.last_real && j == a.nst - 1;
     void* out = a.out[j];
+    if (PAIRS && !real_out) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+      for (int r = 0; r < 4; ++r) {
+        float4* row = reinterpret_cast<float4*>(static_cast<float2*>(out) + size_t(y0 + 4 * ty + r) * nx + (x0 + 4 * tx));
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        if (!(R.outm & (1u << (4 * r + c)))) continue;
-        const size_t g = size_t(y0 + 4 * ty + r) * nx + (x0 + 4 * tx + c);
-        const float uu = halfv(U2[r][c >> 1], c & 1);
-        if (real_out) {
-          static_cast<float*>(out)[g] = uu;
-          if (a.check_finite) bad |= (__float_as_uint(uu) & 0x7f800000u) == 0x7f800000u;
-        } else {
-          static_cast<float2*>(out)[g] = make_float2(uu, halfv(V2[r][c >> 1], c & 1));
-        }
+        for (int h = 0; h < 2; ++h)
+          if (R.outm & (1u << (4 * r + 2 * h))) row[h] = make_float4(U2[r][h].x, V2[r][h].x, U2[r][h].y, V2[r][h].y);
       }
+    } else {
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          if (!(R.outm & (1u << (4 * r + c)))) continue;
+          const size_t g = size_t(y0 + 4 * ty + r) * nx + (x0 + 4 * tx + c);
+          const float uu = halfv(U2[r][c >> 1], c & 1);
+          if (real_out) {
+            static_cast<float*>(out)[g] = uu;
+            if (a.check_finite) bad |= (__float_as_uint(uu) & 0x7f800000u) == 0x7f800000u;
+          } else {
+            static_cast<float2*>(out)[g] = make_float2(uu, halfv(V2[r][c >> 1], c & 1));
+          }
+        }
+    }
   }
   if (bad) atomicOr(a.status, ST_NONFINITE);
 }
@@ -277,7 +302,7 @@ __global__ void __launch_bounds__(RT_THREADS, 2) k_tape_tb2d(const AdjTbArgs a) 
 // ------------------------------------------------------------------------------------------
 // Reverse pass.
 
-template <bool PERIODIC>
+template <bool PERIODIC, bool PAIRS>
 __global__ void __launch_bounds__(RT_THREADS, 2) k_adjrev_tb2d(const AdjTbArgs a) {
   extern __shared__ __align__(16) unsigned char at_smem[];
   RevShared& sh = *reinterpret_cast<RevShared*>(at_smem);
@@ -353,26 +378,39 @@ __global__ void __launch_bounds__(RT_THREADS, 2) k_adjrev_tb2d(const AdjTbArgs a
 
   // lam as horizontal cell pairs: LX[r][h] = (Re lam of cell (r, 2h), of cell (r, 2h + 1))
   float2 LX[4][2], LY[4][2];
+  if (PAIRS && a.l_mode != 0) {
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < 4; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      float lx = 0.f, ly = 0.f;
-      if (PERIODIC || (R.inside & (1u << (4 * r + c)))) {
-        const size_t g = size_t(R.gyr[r]) * nx + R.gxc[c];
-        if (a.l_mode == 1) {
-          const float2 w = static_cast<const float2*>(a.L_in)[g];
-          lx = w.x;
-          ly = w.y;
-        } else if (a.l_mode == 2) {
-          lx = static_cast<const float2*>(a.L_in)[g].x;
-        } else {
-          lx = static_cast<const float*>(a.L_in)[g];
-        }
+      for (int h = 0; h < 2; ++h) {
+        float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (PERIODIC || (R.inside & (1u << (4 * r + 2 * h))))
+          w = *reinterpret_cast<const float4*>(static_cast<const float2*>(a.L_in) + size_t(R.gyr[r]) * nx + R.gxc[2 * h]);
+        LX[r][h] = make_float2(w.x, w.z);
+        LY[r][h] = a.l_mode == 1 ? make_float2(w.y, w.w) : make_float2(0.f, 0.f);
       }
-      set_half(LX[r][c >> 1], c & 1, lx);
-      set_half(LY[r][c >> 1], c & 1, ly);
-    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        float lx = 0.f, ly = 0.f;
+        if (PERIODIC || (R.inside & (1u << (4 * r + c)))) {
+          const size_t g = size_t(R.gyr[r]) * nx + R.gxc[c];
+          if (a.l_mode == 1) {
+            const float2 w = static_cast<const float2*>(a.L_in)[g];
+            lx = w.x;
+            ly = w.y;
+          } else if (a.l_mode == 2) {
+            lx = static_cast<const float2*>(a.L_in)[g].x;
+          } else {
+            lx = static_cast<const float*>(a.L_in)[g];
+          }
+        }
+        set_half(LX[r][c >> 1], c & 1, lx);
+        set_half(LY[r][c >> 1], c & 1, ly);
+      }
+  }
   float dk[4][4];  // dJ/dkappa of each cell over the pass's stages
 #pragma unroll
   for (int r = 0; r < 4; ++r)
@@ -528,15 +566,35 @@ __global__ void __launch_bounds__(RT_THREADS, 2) k_adjrev_tb2d(const AdjTbArgs a
     dk[0][2] += wgt(bS, 2, gs.z);
     dk[0][3] += wgt(bS, 3, gs.w);
   }
+  if constexpr (PAIRS) {
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < 4; ++r) {
+      const size_t g = size_t(y0 + 4 * ty + r) * nx + (x0 + 4 * tx);
+      float4* lo = reinterpret_cast<float4*>(a.L_out + g);
+      double2* dr = reinterpret_cast<double2*>(a.dk + g);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      if (!(R.outm & (1u << (4 * r + c)))) continue;
-      const size_t g = size_t(y0 + 4 * ty + r) * nx + (x0 + 4 * tx + c);
-      a.L_out[g] = make_float2(halfv(LX[r][c >> 1], c & 1), halfv(LY[r][c >> 1], c & 1));
-      if (a.dk) a.dk[g] += double(dk[r][c]);
+      for (int h = 0; h < 2; ++h) {
+        if (!(R.outm & (1u << (4 * r + 2 * h)))) continue;
+        lo[h] = make_float4(LX[r][h].x, LY[r][h].x, LX[r][h].y, LY[r][h].y);
+        if (a.dk) {
+          double2 d = dr[h];
+          d.x += double(dk[r][2 * h]);
+          d.y += double(dk[r][2 * h + 1]);
+          dr[h] = d;
+        }
+      }
     }
+  } else {
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (!(R.outm & (1u << (4 * r + c)))) continue;
+        const size_t g = size_t(y0 + 4 * ty + r) * nx + (x0 + 4 * tx + c);
+        a.L_out[g] = make_float2(halfv(LX[r][c >> 1], c & 1), halfv(LY[r][c >> 1], c & 1));
+        if (a.dk) a.dk[g] += double(dk[r][c]);
+      }
+  }
 }
 
 // Spread over the SMs (500 x 487, s = 32, forward and backward: 1072 -> 852 us), but not where a launch takes less
@@ -546,9 +604,9 @@ size_t adj_spread(size_t need, dim3 grid, const Residency& res) {
   return 3 * regions > res.sms ? spread_smem(need, regions, res.sms, res.per_sm) : need;
 }
 
-template <bool PERIODIC>
+template <bool PERIODIC, bool PAIRS>
 cudaError_t launch_rev(const AdjTbArgs& a, dim3 grid, cudaStream_t st) {
-  const auto kern = k_adjrev_tb2d<PERIODIC>;
+  const auto kern = k_adjrev_tb2d<PERIODIC, PAIRS>;
   static const Residency res = spread_residency(kern, RT_THREADS, sizeof(RevShared), 0);
   if (res.err != cudaSuccess) return res.err;
   {
@@ -569,6 +627,30 @@ cudaError_t launch_rev(const AdjTbArgs& a, dim3 grid, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+template <bool PERIODIC, bool PAIRS>
+cudaError_t launch_tape(const AdjTbArgs& a, dim3 grid, cudaStream_t st) {
+  const auto kern = k_tape_tb2d<PERIODIC, PAIRS>;
+  constexpr size_t fixed = 2 * 2 * 2 * 256 * sizeof(float4);  // its static shared memory
+  static const Residency res = spread_residency(kern, RT_THREADS, 0, fixed);
+  if (res.err != cudaSuccess) return res.err;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(RT_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = adj_spread(fixed, grid, res) - fixed;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a);
+  count_launch();
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// (the tape, lam and dk slots are 256-byte aligned)
+bool adj_pairs(const frkc2_problem& p, int k) { return p.n[0] % 2 == 0 && k % 2 == 0; }
+
 AdjTbArgs base_args(const frkc2_problem& p, int k, int nst, const void* fx, const void* fy, unsigned* status) {
   AdjTbArgs a{};
   a.nx = int(p.n[0]);
@@ -588,6 +670,40 @@ dim3 region_grid(const frkc2_problem& p, int k) {
 
 }  // namespace
 
+// Stages of a tape (rev = false) or reverse pass: 8, or for pair access the even count whose passes take the
+// least by a model of their time in us fitted to measurements (k = 4 .. 12, periodic grids of 100^2 to 1500^2): a
+// wave with one or two regions an SM, waves overlapping by c at their ends.  Model / measured: reverse 1024^2
+// k = 8 79 / 78, k = 10 89 / 93; tape 1024^2 k = 8 35 / 32, k = 10 39 / 38, 300 x 277 k = 12 15.8 / 16.2.
+int adj_tb2d_k(const frkc2_problem& p, int s, bool rev) {
+  if (!adj_pairs(p, 8)) return 8;
+  static const int sms = [] {
+    int dev = 0, n = 152;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      n = 152;
+    return n;
+  }();
+  auto pass = [&](int k) {
+    const dim3 g = region_grid(p, k);
+    const long long regions = (long long)g.x * g.y, slots = 2ll * sms, full = regions / slots, rest = regions % slots;
+    auto wave = [&](long long ctas) {
+      if (rev) return ctas > sms ? 22.0 + 2.45 * k : 13.0 + 1.75 * k;
+      return ctas > sms ? 12.4 + 0.97 * k : 8.0 + 0.65 * k;
+    };
+    const double c = rev ? 4.0 : 5.5;
+    return double(full) * (wave(slots) - c) + (rest ? wave(rest) : c);
+  };
+  int best = 8;
+  double least = 0.0;
+  for (int k = 4; k <= 12; k += 2) {
+    const double us = (s / k) * pass(k) + (s % k ? pass(s % k) : 0.0);
+    if (k == 4 || us < least) {
+      best = k;
+      least = us;
+    }
+  }
+  return best;
+}
+
 bool adj_tb2d_supported(const frkc2_problem& p, int k) {
   return p.ndim == 2 && p.precision == FRKC2_FP32 && p.kappa_kind != FRKC2_KAPPA_POWER && k >= 1 &&
          k <= AT_KMAX && 2 * k < RT_R && p.n[0] * p.n[1] < (int64_t(1) << 31);
@@ -606,28 +722,9 @@ cudaError_t launch_tape_tb2d(const frkc2_problem& p, int k, const AdjTbPass& t, 
     a.cb[j] = float(t.cb[j]);
   }
   const dim3 grid = region_grid(p, k);
-  const auto tk = p.bc == FRKC2_BC_PERIODIC ? k_tape_tb2d<true> : k_tape_tb2d<false>;
-  constexpr size_t fixed = 2 * 2 * 2 * 256 * sizeof(float4);  // its static shared memory
-  static const Residency res_p = spread_residency(k_tape_tb2d<true>, RT_THREADS, 0, fixed);
-  static const Residency res_d = spread_residency(k_tape_tb2d<false>, RT_THREADS, 0, fixed);
-  const Residency& res = p.bc == FRKC2_BC_PERIODIC ? res_p : res_d;
-  if (res.err != cudaSuccess) return res.err;
-  {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(RT_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = adj_spread(fixed, grid, res) - fixed;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    const cudaError_t le = cudaLaunchKernelEx(&cfg, tk, a);
-    if (le != cudaSuccess) return le;
-  }
-  count_launch();
-  return cudaGetLastError();
+  const bool pairs = adj_pairs(p, k);
+  if (p.bc == FRKC2_BC_PERIODIC) return pairs ? launch_tape<true, true>(a, grid, st) : launch_tape<true, false>(a, grid, st);
+  return pairs ? launch_tape<false, true>(a, grid, st) : launch_tape<false, false>(a, grid, st);
 }
 
 cudaError_t launch_adjrev_tb2d(const frkc2_problem& p, int k, const AdjTbPass& t, const void* fx, const void* fy,
@@ -645,7 +742,9 @@ cudaError_t launch_adjrev_tb2d(const frkc2_problem& p, int k, const AdjTbPass& t
     a.cb[j] = float(t.cb[j]);
   }
   const dim3 grid = region_grid(p, k);
-  return p.bc == FRKC2_BC_PERIODIC ? launch_rev<true>(a, grid, st) : launch_rev<false>(a, grid, st);
+  const bool pairs = adj_pairs(p, k);
+  if (p.bc == FRKC2_BC_PERIODIC) return pairs ? launch_rev<true, true>(a, grid, st) : launch_rev<true, false>(a, grid, st);
+  return pairs ? launch_rev<false, true>(a, grid, st) : launch_rev<false, false>(a, grid, st);
 }
 
 }  // namespace frkc2

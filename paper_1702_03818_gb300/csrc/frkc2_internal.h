@@ -121,6 +121,8 @@ struct TbShape {
   double us;
 };
 TbShape tb2d_shape(int nx, int ny, int s);
+// 64 x 64 regions and an even k: a cell's column keeps its parity in its thread, and with it its rounding
+TbShape tb2d_shape_even(int nx, int ny, int s);
 bool small1d_supported(const frkc2_problem& p, int s);
 // 2D FP32 wavefront pass (pass_wf2d.cu): CTAs of WF_NW warps stream column strips of
 // 64 WF_NW cells up the grid with up to WF_KMAX stage levels in flight; rows arrive by TMA.
@@ -184,6 +186,7 @@ struct AdjTbPass {
   double ca[16], cb[16];  // dt a_l / dx^2 of stage j
 };
 bool adj_tb2d_supported(const frkc2_problem& p, int k);
+int adj_tb2d_k(const frkc2_problem& p, int s, bool rev);  // stages of a tape or reverse pass
 cudaError_t launch_tape_tb2d(const frkc2_problem& p, int k, const AdjTbPass& t, const void* fx, const void* fy,
                              unsigned* status, cudaStream_t st);
 cudaError_t launch_adjrev_tb2d(const frkc2_problem& p, int k, const AdjTbPass& t, const void* fx, const void* fy,

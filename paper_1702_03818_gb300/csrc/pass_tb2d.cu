@@ -307,29 +307,31 @@ static double tb2d_pass_us(int C, int k, long long regions, int sms) {
   return double(full) * (wave(slots) - c) + (rest ? wave(rest) : c);
 }
 
-static TbShape tb2d_best(int C, int nx, int ny, int s, int kmax) {
+static TbShape tb2d_best(int C, int nx, int ny, int s, int kmin, int kstep, int kmax) {
   static const int sms = [] {
     int dev = 0, n = 152;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       n = 152;
     return n;
   }();
-  TbShape best{C, 1, 0.0};
-  for (int k = 1; k <= std::min(s, kmax); ++k) {
+  TbShape best{C, kmin, 0.0};
+  for (int k = kmin; k <= std::min(s, kmax); k += kstep) {
     auto pass = [&](int q) {
       const int T = 16 * C - 2 * q;
       return tb2d_pass_us(C, q, (long long)((nx + T - 1) / T) * ((ny + T - 1) / T), sms);
     };
     const double us = (s / k) * pass(k) + (s % k ? pass(s % k) : 0.0);
-    if (k == 1 || us < best.us) best = TbShape{C, k, us};
+    if (k == kmin || us < best.us) best = TbShape{C, k, us};
   }
   return best;
 }
 
 TbShape tb2d_shape(int nx, int ny, int s) {
-  const TbShape a = tb2d_best(2, nx, ny, s, 10), b = tb2d_best(4, nx, ny, s, 12);
+  const TbShape a = tb2d_best(2, nx, ny, s, 1, 1, 10), b = tb2d_best(4, nx, ny, s, 1, 1, 12);
   return a.us < b.us ? a : b;
 }
+
+TbShape tb2d_shape_even(int nx, int ny, int s) { return tb2d_best(4, nx, ny, s, 2, 2, 12); }
 
 bool tb2d_supported(const frkc2_problem& p, int k) {
   return p.ndim == 2 && p.precision == FRKC2_FP32 && p.kappa_kind != FRKC2_KAPPA_POWER && k >= 1 && 2 * k < 64;
