@@ -454,7 +454,7 @@ bool run_segment_plain_tb(const AdjCtx& C, int j) {
       }
       a.in_mode = curV ? PASS_IO_PLANAR : PASS_IO_REAL;
       a.out_mode = outV ? PASS_IO_PLANAR : PASS_IO_REAL;
-      if (launch_pass_tb2d(p, a, C.st, q > 0 || ps > 0, shape.cells) != cudaSuccess) return false;
+      if (launch_pass_tb2d(p, a, TbIo{nullptr, nullptr, 0, a.nx, a.nx}, C.st, q > 0 || ps > 0, shape.cells) != cudaSuccess) return false;
       curU = outU;
       curV = outV;
     }

@@ -229,11 +229,18 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
     if (!wf_ok) return FRKC2_EUNSUPPORTED;
     use_wf = true;
   } else if (kern == 0) {
-    // FP32 k-stage passes: the wavefront where it recomputes fewer cells than the 64 x 64 regions,
-    // allowing for its 8 % higher cost per computed cell-stage (measured at 2048^2, k = 8)
+    // FP32 k-stage passes.  The library's choice is the cheaper by the two models of a step: the regions up to
+    // about 3000^2, the wavefront above (2048^2 6.28 against 7.26 us a stage, 4096^2 23.0 against 22.6).  For a
+    // given k, the wavefront where it recomputes fewer cells than the 64 x 64 regions, allowing for its 8 %
+    // higher cost per computed cell-stage (2048^2, k = 8, single-cell accesses in the regions).
+    const int nx = int(p.n[0]), ny = int(p.n[1]);
+    const bool choose = tb_ok && k > 1 && !(tune && tune->k);
+    const TbShape sh = choose ? tb2d_shape(nx, ny, plan->s) : TbShape{4, k, 0.0};
     bool wf_wins = false;
-    if (wf_ok && tb_ok && k > 1) {
-      const int T = 64 - 2 * k, nx = int(p.n[0]), ny = int(p.n[1]);
+    if (wf_ok && choose) {
+      wf_wins = k == 8 && (plan->s + 7) / 8 * wf2d_pass8_us(nx, ny) < sh.us;
+    } else if (wf_ok && tb_ok && k > 1) {
+      const int T = 64 - 2 * k;
       const double regions = double((nx + T - 1) / T) * ((ny + T - 1) / T) * 64.0 * 64.0 / (double(nx) * ny);
       wf_wins = 1.08 * wf2d_recompute(nx, ny, k) < regions;
     }
@@ -241,11 +248,8 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
       use_wf = true;
     } else if (tb_ok && k > 1) {
       use_tb = true;
-      if (!(tune && tune->k)) {  // the library's choice of region size and stages per pass
-        const TbShape sh = tb2d_shape(int(p.n[0]), int(p.n[1]), plan->s);
-        tb_cells = sh.cells;
-        k = sh.k;
-      }
+      tb_cells = sh.cells;
+      k = sh.k;
     } else if (stream3d_ok) {
       use_stream3d = true;
     } else {
@@ -271,7 +275,7 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* base = static_cast<char*>(ws);
-  if (p.kappa_kind != FRKC2_KAPPA_POWER && !use_stream3d) {  // (the 3D streaming pass reads the cells')
+  if (p.kappa_kind != FRKC2_KAPPA_POWER && !use_stream3d && !use_tb) {  // (these two take the conductivities in other forms)
     if (launch_faces(p, base + L.fx, base + L.fy, base + L.fz, st) != cudaSuccess) return FRKC2_ECUDA;
   }
   void* ua = base + L.ua;
@@ -405,6 +409,57 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
       return FRKC2_ECUDA;
     return FRKC2_OK;
   }
+  if (use_tb) {
+    // Rows padded to a multiple of 4 cells, so that the passes move whole vectors: the faces in the face-pair
+    // slot; the state buffers, where nx is not such a multiple, with the first in the place of the unpadded faces.
+    const int nx = a.nx, ny = a.ny, fpitch = (nx + 1 + 3) / 4 * 4;
+    float* fxp = reinterpret_cast<float*>(base + L.fen);
+    const TbIo faces{fxp, fxp + size_t(ny) * fpitch, fpitch, 0, 0};
+    if (launch_faces_padded(p, fxp, fxp + size_t(ny) * fpitch, fpitch, st) != cudaSuccess) return FRKC2_ECUDA;
+    int pitch = nx;
+    const int np = (nx + 3) / 4 * 4;
+    const size_t buf = align256(size_t(ny) * np * sizeof(float));
+    if (np != nx && L.fx + buf <= L.fen && L.ua + 3 * buf <= L.total) {
+      pitch = np;
+      ua = base + L.fx;
+      va = base + L.ua;
+      ub = base + L.ua + buf;
+      vb = base + L.ua + 2 * buf;
+    }
+    for (int n = 0; n < nsteps; ++n) {
+      const NvtxRange step_range("frkc2 step");
+      for (int q = 0; q < npass; ++q) {
+        const NvtxRange pass_range("frkc2 pass");
+        const int l0 = q * k, kq = std::min(k, s - l0);
+        const bool last = q == npass - 1;
+        // a pass never writes the array it reads: with one pass per step the real state alternates between u and ua
+        void* outU = last && curU != u ? u : (curU == ua ? ub : ua);
+        void* outV = last ? nullptr : (curV == va ? vb : va);
+        a.k = kq;
+        a.U_in = curU;
+        a.V_in = curV;
+        a.U_out = outU;
+        a.V_out = outV;
+        a.check_finite = last ? 1 : 0;
+        for (int j = 0; j < kq; ++j) {
+          a.caf[j] = float(dt * plan->a_re[l0 + j] / h2);
+          a.cbf[j] = float(dt * plan->a_im[l0 + j] / h2);
+        }
+        TbIo io = faces;
+        io.in_pitch = curU == u ? nx : pitch;
+        io.out_pitch = outU == u ? nx : pitch;
+        // passes after the first may start while the previous one drains (the faces, written before the
+        // first pass, are read before the wait for the previous pass)
+        if (launch_pass_tb2d(p, a, io, st, n > 0 || q > 0, tb_cells) != cudaSuccess) return FRKC2_ECUDA;
+        curU = outU;
+        curV = outV;
+      }
+    }
+    if (curU != u && cudaMemcpy2DAsync(u, size_t(nx) * sizeof(float), curU, size_t(pitch) * sizeof(float), size_t(nx) * sizeof(float),
+                                       size_t(ny), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+      return FRKC2_ECUDA;
+    return FRKC2_OK;
+  }
   if (use_stream2d || use_stream3d) {
     // interleaved complex state between passes: W buffers at ua (with va) and ub (with vb)
     if (use_stream2d && launch_face_pairs(p, base + L.fx, base + L.fy, base + L.fen, st) != cudaSuccess)
@@ -468,10 +523,7 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
       }
       a.in_mode = curV ? PASS_IO_PLANAR : PASS_IO_REAL;
       a.out_mode = outV ? PASS_IO_PLANAR : PASS_IO_REAL;
-      // passes after the first may start while the previous one drains (face conductivities,
-      // written before the first pass, are read before the wait for the previous pass)
-      const cudaError_t e = use_tb ? launch_pass_tb2d(p, a, st, n > 0 || q > 0, tb_cells) : launch_pass_generic(p, a, st);
-      if (e != cudaSuccess) return FRKC2_ECUDA;
+      if (launch_pass_generic(p, a, st) != cudaSuccess) return FRKC2_ECUDA;
       curU = outU;
       curV = outV;
     }

@@ -65,6 +65,25 @@ __global__ void k_faces(const FaceArgs a) {
   }
 }
 
+// The 2D FP32 faces in rows of `pitch`: x face i of row y at fxp[y pitch + i] (i = 0 .. nx), y face j of column x at
+// fyp[j pitch + x] (j = 0 .. ny).
+__global__ void k_faces_padded(const FaceArgs a, float* __restrict__ fxp, float* __restrict__ fyp, int pitch) {
+  const float* K = static_cast<const float*>(a.kappa);
+  const bool periodic = a.bc == FRKC2_BC_PERIODIC;
+  const bool cst = a.kind == FRKC2_KAPPA_CONST;
+  const size_t nfx = size_t(a.ny) * pitch, total = nfx + size_t(a.ny + 1) * pitch;
+  for (size_t t = blockIdx.x * size_t(blockDim.x) + threadIdx.x; t < total; t += size_t(gridDim.x) * blockDim.x) {
+    const bool isx = t < nfx;
+    const size_t q = isx ? t : t - nfx;
+    const int row = int(q / pitch), i = int(q % pitch);
+    if (isx) {
+      fxp[q] = i > a.nx ? 0.f : cst ? float(a.c) : face_value<float>(K, i, a.nx, size_t(row) * a.nx, 1, periodic);
+    } else {
+      fyp[q] = i >= a.nx ? 0.f : cst ? float(a.c) : face_value<float>(K, row, a.ny, size_t(i), size_t(a.nx), periodic);
+    }
+  }
+}
+
 struct RhoArgs {
   int ndim, bc, kind;
   int nx, ny, nz;
@@ -168,6 +187,15 @@ cudaError_t launch_faces(const frkc2_problem& p, void* fx, void* fy, void* fz, c
     k_faces<double><<<grid_for(total, threads), threads, 0, st>>>(a);
   else
     k_faces<float><<<grid_for(total, threads), threads, 0, st>>>(a);
+  count_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_faces_padded(const frkc2_problem& p, float* fxp, float* fyp, int pitch, cudaStream_t st) {
+  FaceArgs a{p.ndim, p.bc, p.kappa_kind, int(p.n[0]), int(p.n[1]), int(p.n[2]), p.kappa_c,
+             p.kappa, nullptr, nullptr, nullptr};
+  const int threads = 256;
+  k_faces_padded<<<grid_for(size_t(2 * p.n[1] + 1) * pitch, threads), threads, 0, st>>>(a, fxp, fyp, pitch);
   count_launch();
   return cudaGetLastError();
 }

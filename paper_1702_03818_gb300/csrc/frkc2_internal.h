@@ -113,8 +113,15 @@ cudaError_t launch_face_pairs(const frkc2_problem& p, const void* fx, const void
 // overlap_previous: the launch may start while the previous launch on the stream (a pass of
 // the same kind) finishes; its CTAs read the pass input only after that launch completes.
 // cells: a thread's cells along each axis, 4 (64 x 64 regions) or 2 (32 x 32, k < 16)
-cudaError_t launch_pass_tb2d(const frkc2_problem& p, const PassArgs& a, cudaStream_t st, bool overlap_previous,
-                             int cells = 4);
+struct TbIo {
+  const float* fxp;  // x faces [ny][fpitch], y faces [ny + 1][fpitch] in rows padded to a multiple of 4 (launch_faces_padded),
+  const float* fyp;  // or nullptr: the unpadded arrays of PassArgs
+  int fpitch;
+  int in_pitch, out_pitch;  // row pitch of the state read and written
+};
+cudaError_t launch_pass_tb2d(const frkc2_problem& p, const PassArgs& a, const TbIo& io, cudaStream_t st,
+                             bool overlap_previous, int cells = 4);
+cudaError_t launch_faces_padded(const frkc2_problem& p, float* fxp, float* fyp, int pitch, cudaStream_t st);
 // region size and stages per pass for a grid and a plan of s stages, with the model's us a step
 struct TbShape {
   int cells, k;
@@ -130,6 +137,7 @@ constexpr int WF_NW = 4;
 int wf2d_face_pitch(int nx);
 // computed / output cell-stages of the wavefront pass at its default launch
 double wf2d_recompute(int nx, int ny, int k);
+double wf2d_pass8_us(int nx, int ny);
 // k stages per pass and s stages per step: every pass (the last may be shorter) needs an
 // instantiated stage count (1, 2, 4, 6, 8, 10 or 12)
 bool wf2d_supported(const frkc2_problem& p, int k, int s, const void* u);

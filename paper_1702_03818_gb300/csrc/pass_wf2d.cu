@@ -476,6 +476,9 @@ bool wf2d_k_supported(int k) { return k == 1 || k == 2 || k == 4 || k == 6 || k 
 
 int wf2d_face_pitch(int nx) { return nx + 4; }
 
+// us of a pass at k = 8 and its default launch: 8.8 ps a computed cell (2048^2 58.1, 3000^2 102.8, 4096^2 180.7 measured)
+double wf2d_pass8_us(int nx, int ny) { return 8.8e-6 * double(nx) * ny * wf2d_recompute(nx, ny, 8); }
+
 double wf2d_recompute(int nx, int ny, int k) {
   // strips of 256 columns with 2h halo columns; one wave of 3 CTAs per SM (the occupancy of the
   // k <= 8 instantiations); chunks of H rows in which every level runs H + 2k rows
