@@ -275,7 +275,7 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* base = static_cast<char*>(ws);
-  if (p.kappa_kind != FRKC2_KAPPA_POWER && !use_stream3d && !use_tb) {  // (these two take the conductivities in other forms)
+  if (p.kappa_kind != FRKC2_KAPPA_POWER && !use_stream3d && !use_tb && !use_tb_df) {  // (these take the conductivities in other forms)
     if (launch_faces(p, base + L.fx, base + L.fy, base + L.fz, st) != cudaSuccess) return FRKC2_ECUDA;
   }
   void* ua = base + L.ua;
@@ -338,7 +338,24 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
     return FRKC2_OK;
   }
   if (use_tb_df) {
-    // float-pair state (float4 per cell) between passes, in the ua (with va) and ub (with vb) slots
+    // The workspace from the face slots on: faces in padded rows, then two pair states of four padded planes
+    // each (the unpadded faces and face pairs, which this pass does not use, leave the room).
+    // (Narrow grids whose padding does not fit keep their rows as they are and move single cells.)
+    const int nx = a.nx, ny = a.ny;
+    int fpitch = (nx + 1 + 3) / 4 * 4, pitch = (nx + 3) / 4 * 4;
+    auto faces_bytes = [&] { return align256(size_t(2 * ny + 1) * fpitch * sizeof(float)); };
+    auto state_bytes4 = [&] { return align256(4 * size_t(ny) * pitch * sizeof(float)); };
+    if (L.fx + faces_bytes() + 2 * state_bytes4() > L.total) {
+      fpitch = nx + 1;
+      pitch = nx;
+    }
+    const size_t plane = size_t(ny) * pitch, faces = faces_bytes(), buf = state_bytes4();
+    float* fxp = reinterpret_cast<float*>(base + L.fx);
+    if (launch_faces_padded(p, fxp, fxp + size_t(ny) * fpitch, fpitch, st) != cudaSuccess) return FRKC2_ECUDA;
+    a.fx = fxp;
+    a.fy = fxp + size_t(ny) * fpitch;
+    ua = base + L.fx + faces;
+    ub = base + L.fx + faces + buf;
     // a pass never writes the array it reads (its regions' halos overlap other CTAs' output
     // tiles): with one pass per step the real state alternates between u and ua
     for (int n = 0; n < nsteps; ++n) {
@@ -363,7 +380,7 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
           a.caf[j] = float(a.ca[j]);
           a.cbf[j] = float(a.cb[j]);
         }
-        if (launch_pass_tb2d_df(p, a, st, n > 0 || q > 0) != cudaSuccess) return FRKC2_ECUDA;
+        if (launch_pass_tb2d_df(p, a, fpitch, pitch, plane, st, n > 0 || q > 0) != cudaSuccess) return FRKC2_ECUDA;
         curU = outU;
       }
     }

@@ -393,7 +393,7 @@ __device__ __noinline__ bool df_region_call(DfShared& sh, int nx, int ny, int k,
     ca = float(cf[2 * j]);
     cb = float(cf[2 * j + 1]);
   };
-  return tb2d_df_region<PERIODIC, IN_REAL, OUT_REAL, true>(sh, nx, ny, k, kq, x0, y0, in, out, FX, FY, coef, true,
+  return tb2d_df_region<PERIODIC, IN_REAL, OUT_REAL, true, false>(sh, nx, ny, k, kq, x0, y0, in, out, FX, FY, coef, true,
                                                           [] {});
 }
 

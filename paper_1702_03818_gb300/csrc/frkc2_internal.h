@@ -154,7 +154,10 @@ int stream3d_chunks(long long blocks, int nz, long long slots);
 bool stream3d_supported(const frkc2_problem& p);
 cudaError_t launch_pass_stream3d_f32(const frkc2_problem& p, const PassArgs& a, cudaStream_t st);
 cudaError_t launch_pass_stream3d(const frkc2_problem& p, const PassArgs& a, cudaStream_t st);
-cudaError_t launch_pass_tb2d_df(const frkc2_problem& p, const PassArgs& a, cudaStream_t st, bool overlap_previous);
+// faces in padded rows (a.fx, a.fy of pitch fpitch), the pair state between passes as four planes of `plane` floats in
+// rows of `pitch` (both pitches and the plane multiples of 4)
+cudaError_t launch_pass_tb2d_df(const frkc2_problem& p, const PassArgs& a, int fpitch, int pitch, size_t plane, cudaStream_t st,
+                                bool overlap_previous);
 cudaError_t launch_pass_stream2d_df(const frkc2_problem& p, const PassArgs& a, const void* fen, cudaStream_t st);
 cudaError_t launch_pass_paired2d(const frkc2_problem& p, const PassArgs& a, const void* fen, cudaStream_t st);
 bool tb2d_supported(const frkc2_problem& p, int k);

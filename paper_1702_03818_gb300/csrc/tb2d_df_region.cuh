@@ -15,7 +15,7 @@
 // and all of it but the x differences and x flux terms as packed two-lane instructions (add /
 // fma .f32x2 of the sm_100 family) on two cells at once.  IN_REAL: the state comes as the
 // double real state and is split; OUT_REAL: hi + lo goes out as a double; in between the state
-// is one float4 (Uh, Ul, Vh, Vl) per cell, as in the DFLOAT streaming pass.
+// is one float4 (Uh, Ul, Vh, Vl) per cell, as in the DFLOAT streaming pass, or four planes (PLANAR).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -57,11 +57,19 @@ __device__ __forceinline__ float half_of(float2 a, int i) { return i ? a.y : a.x
 // single-problem pass waits there for the previous pass).  L1BYPASS: state loads through L2
 // (buffers other CTAs of the same launch wrote).  Returns true if a stored value is not finite
 // (when check_finite; OUT_REAL only).
-template <bool PERIODIC, bool IN_REAL, bool OUT_REAL, bool L1BYPASS, class Coef, class AfterFaces>
+// PLANAR: faces in padded rows (FX, FY of pitch io.fpitch, launch_faces_padded) and the pair state as four planes
+// (Uh, Ul, Vh, Vl) of io.plane floats in rows of io.pitch; where both pitches are multiples of 4 a thread's rows move as whole
+// vectors, neighbouring threads' next to each other (a float4 per cell puts them 64 bytes apart).
+struct DfIo {
+  int fpitch, pitch;
+  size_t plane;
+};
+
+template <bool PERIODIC, bool IN_REAL, bool OUT_REAL, bool L1BYPASS, bool PLANAR, class Coef, class AfterFaces>
 __device__ __forceinline__ bool tb2d_df_region(DfShared& sh, int nx, int ny, int k, int kq, int x0, int y0,
                                                const void* in, void* out, const float* __restrict__ FX,
                                                const float* __restrict__ FY, Coef coef, bool check_finite,
-                                               AfterFaces after_faces) {
+                                               AfterFaces after_faces, const DfIo io = DfIo{}) {
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   float4* myfx = &sh.fx4[0][tid];  // row r at myfx[r * RT_THREADS]
   float4* myfy = &sh.fy4[0][tid];
@@ -78,54 +86,102 @@ __device__ __forceinline__ bool tb2d_df_region(DfShared& sh, int nx, int ny, int
   }
   unsigned inside = 0;
 #pragma unroll
-  for (int r = 0; r < 5; ++r) {
-    float fxr[5], fyr[4];
+  for (int r = 0; r < 4; ++r)
 #pragma unroll
-    for (int c = 0; c < 5; ++c) {
-      if (r < 4) {  // x face c of row r
-        float v = 0.f;
-        if (PERIODIC || (yin[r] && gxc[c] >= 0 && gxc[c] <= nx)) v = FX[size_t(gyr[r]) * (nx + 1) + gxc[c]];
-        fxr[c] = v;
-      }
-      if (c < 4) {  // y face r of column c
-        float v = 0.f;
-        if (PERIODIC || (xin[c] && gyr[r] >= 0 && gyr[r] <= ny)) v = FY[size_t(gyr[r]) * nx + gxc[c]];
-        fyr[c] = v;
-        if (r < 4 && xin[c] && yin[r]) inside |= 1u << (4 * r + c);
+    for (int c = 0; c < 4; ++c)
+      if (xin[c] && yin[r]) inside |= 1u << (4 * r + c);
+  const int pfx = PLANAR ? io.fpitch : nx + 1, pfy = PLANAR ? io.fpitch : nx;
+  // the thread's rows lie in the grid in one piece (not across the periodic wrap) and aligned
+  const bool rows4 = PLANAR && ((io.pitch | io.fpitch) & 3) == 0;
+  const bool run = rows4 && (gxc[0] & 3) == 0 && gxc[3] == gxc[0] + 3 && (PERIODIC || (xin[0] && xin[3]));
+  if (PLANAR && run) {
+#pragma unroll
+    for (int r = 0; r < 5; ++r) {
+      float4 fyv = make_float4(0.f, 0.f, 0.f, 0.f), fxv = fyv;
+      if (PERIODIC || (gyr[r] >= 0 && gyr[r] <= ny)) fyv = *reinterpret_cast<const float4*>(FY + size_t(gyr[r]) * pfy + gxc[0]);
+      myfy[r * RT_THREADS] = fyv;
+      if (r < 4) {
+        if (PERIODIC || yin[r]) {
+          const float* q = FX + size_t(gyr[r]) * pfx + gxc[0];
+          const float4 v = *reinterpret_cast<const float4*>(q);
+          fxv = make_float4(v.y, v.z, v.w, q[4]);  // (periodic face nx repeats face 0)
+        }
+        myfx[r * RT_THREADS] = fxv;
       }
     }
-    // face 0 of a row is the west neighbour's face 4: its flux term comes from there
-    if (r < 4) myfx[r * RT_THREADS] = make_float4(fxr[1], fxr[2], fxr[3], fxr[4]);
-    myfy[r * RT_THREADS] = make_float4(fyr[0], fyr[1], fyr[2], fyr[3]);
+  } else {
+#pragma unroll
+    for (int r = 0; r < 5; ++r) {
+      float fxr[5], fyr[4];
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {
+        if (r < 4) {  // x face c of row r
+          float v = 0.f;
+          if (PERIODIC || (yin[r] && gxc[c] >= 0 && gxc[c] <= nx)) v = FX[size_t(gyr[r]) * pfx + gxc[c]];
+          fxr[c] = v;
+        }
+        if (c < 4) {  // y face r of column c
+          float v = 0.f;
+          if (PERIODIC || (xin[c] && gyr[r] >= 0 && gyr[r] <= ny)) v = FY[size_t(gyr[r]) * pfy + gxc[c]];
+          fyr[c] = v;
+        }
+      }
+      // face 0 of a row is the west neighbour's face 4: its flux term comes from there
+      if (r < 4) myfx[r * RT_THREADS] = make_float4(fxr[1], fxr[2], fxr[3], fxr[4]);
+      myfy[r * RT_THREADS] = make_float4(fyr[0], fyr[1], fyr[2], fyr[3]);
+    }
   }
   after_faces();
   // the state as horizontal cell pairs: Uh[r][h] = (Uh of cell (r, 2h), of cell (r, 2h + 1))
   float2 Uh[4][2], Ul[4][2], Vh[4][2], Vl[4][2];
+  if (PLANAR && !IN_REAL && run) {
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < 4; ++r) {
+      float4 v[4];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float4 w[2];
+      for (int i = 0; i < 4; ++i) {
+        v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (PERIODIC || yin[r])
+          v[i] = *reinterpret_cast<const float4*>(static_cast<const float*>(in) + i * io.plane + size_t(gyr[r]) * io.pitch + gxc[0]);
+      }
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int c = 2 * h + i;
-        w[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (PERIODIC || (inside & (1u << (4 * r + c)))) {
-          const size_t g = size_t(gyr[r]) * nx + gxc[c];
-          if (IN_REAL) {
-            const double u = L1BYPASS ? __ldcg(static_cast<const double*>(in) + g) : static_cast<const double*>(in)[g];
-            w[i].x = __double2float_rn(u);
-            w[i].y = __double2float_rn(u - double(w[i].x));
-          } else {
-            w[i] = L1BYPASS ? __ldcg(static_cast<const float4*>(in) + g) : static_cast<const float4*>(in)[g];
+      for (int h = 0; h < 2; ++h) {
+        Uh[r][h] = pair_of(v[0], h);
+        Ul[r][h] = pair_of(v[1], h);
+        Vh[r][h] = pair_of(v[2], h);
+        Vl[r][h] = pair_of(v[3], h);
+      }
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float4 w[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const int c = 2 * h + i;
+          w[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (PERIODIC || (inside & (1u << (4 * r + c)))) {
+            const size_t g = size_t(gyr[r]) * (PLANAR && !IN_REAL ? io.pitch : nx) + gxc[c];
+            if (IN_REAL) {
+              const double u = L1BYPASS ? __ldcg(static_cast<const double*>(in) + g) : static_cast<const double*>(in)[g];
+              w[i].x = __double2float_rn(u);
+              w[i].y = __double2float_rn(u - double(w[i].x));
+            } else if (PLANAR) {
+              const float* q = static_cast<const float*>(in) + g;
+              w[i] = make_float4(q[0], q[io.plane], q[2 * io.plane], q[3 * io.plane]);
+            } else {
+              w[i] = L1BYPASS ? __ldcg(static_cast<const float4*>(in) + g) : static_cast<const float4*>(in)[g];
+            }
           }
         }
+        Uh[r][h] = make_float2(w[0].x, w[1].x);
+        Ul[r][h] = make_float2(w[0].y, w[1].y);
+        Vh[r][h] = make_float2(w[0].z, w[1].z);
+        Vl[r][h] = make_float2(w[0].w, w[1].w);
       }
-      Uh[r][h] = make_float2(w[0].x, w[1].x);
-      Ul[r][h] = make_float2(w[0].y, w[1].y);
-      Vh[r][h] = make_float2(w[0].z, w[1].z);
-      Vl[r][h] = make_float2(w[0].w, w[1].w);
-    }
+  }
 
   const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int j = 0; j < kq; ++j) {
@@ -227,22 +283,37 @@ __device__ __forceinline__ bool tb2d_df_region(DfShared& sh, int nx, int ny, int
   }
 
   bool bad = false;
+  const bool vout = rows4 && !OUT_REAL && ((x0 + 4 * tx) & 3) == 0 && 4 * tx >= k && 4 * tx + 4 <= RT_R - k && x0 + 4 * tx + 4 <= nx;
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     const int ry = 4 * ty + r;
     const int gy = y0 + ry;
     if (ry < k || ry >= RT_R - k || gy >= ny) continue;
+    if (PLANAR && vout) {
+      float* q = static_cast<float*>(out) + size_t(gy) * io.pitch + (x0 + 4 * tx);
+      *reinterpret_cast<float4*>(q) = make_float4(Uh[r][0].x, Uh[r][0].y, Uh[r][1].x, Uh[r][1].y);
+      *reinterpret_cast<float4*>(q + io.plane) = make_float4(Ul[r][0].x, Ul[r][0].y, Ul[r][1].x, Ul[r][1].y);
+      *reinterpret_cast<float4*>(q + 2 * io.plane) = make_float4(Vh[r][0].x, Vh[r][0].y, Vh[r][1].x, Vh[r][1].y);
+      *reinterpret_cast<float4*>(q + 3 * io.plane) = make_float4(Vl[r][0].x, Vl[r][0].y, Vl[r][1].x, Vl[r][1].y);
+      continue;
+    }
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const int rx = 4 * tx + c;
       const int gx = x0 + rx;
       if (rx < k || rx >= RT_R - k || gx >= nx) continue;
-      const size_t g = size_t(gy) * nx + gx;
+      const size_t g = size_t(gy) * (PLANAR && !OUT_REAL ? io.pitch : nx) + gx;
       const int h = c >> 1, i = c & 1;
       if (OUT_REAL) {
         const double u = double(half_of(Uh[r][h], i)) + double(half_of(Ul[r][h], i));
         static_cast<double*>(out)[g] = u;
         if (check_finite) bad |= (__double2hiint(u) & 0x7ff00000) == 0x7ff00000;
+      } else if (PLANAR) {
+        float* q = static_cast<float*>(out) + g;
+        q[0] = half_of(Uh[r][h], i);
+        q[io.plane] = half_of(Ul[r][h], i);
+        q[2 * io.plane] = half_of(Vh[r][h], i);
+        q[3 * io.plane] = half_of(Vl[r][h], i);
       } else {
         static_cast<float4*>(out)[g] =
             make_float4(half_of(Uh[r][h], i), half_of(Ul[r][h], i), half_of(Vh[r][h], i), half_of(Vl[r][h], i));
@@ -251,7 +322,5 @@ __device__ __forceinline__ bool tb2d_df_region(DfShared& sh, int nx, int ny, int
   }
   return bad;
 }
-
-
 
 }  // namespace frkc2
