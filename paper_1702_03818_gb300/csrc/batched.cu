@@ -62,6 +62,7 @@ struct BProb {
   void* ub;
   void* vb;
   const double* coef;  // (ca, cb) per stage, dt a_l / dx^2
+  int pitch, fpitch;   // FP32 regions: rows of the workspace state and of the faces, padded to a multiple of 4
 };
 
 struct BHeader {
@@ -401,12 +402,14 @@ __device__ __noinline__ bool df_region_call(DfShared& sh, int nx, int ny, int k,
 template <bool PERIODIC>
 __device__ __noinline__ bool fp32_region_call(RegionShared& sh, int nx, int ny, int k, int kq, int x0, int y0,
                                               const float* Uin, const float* Vin, float* Uout, float* Vout,
-                                              const float* FX, const float* FY, const double* cf) {
+                                              const float* FX, const float* FY, int pf, int pin, int pout,
+                                              const double* cf) {
   auto coef = [&](int j, float& ca, float& cb) {
     ca = float(cf[2 * j]);
     cb = float(cf[2 * j + 1]);
   };
-  return tb2d_region<PERIODIC, true>(sh, nx, ny, k, kq, x0, y0, Uin, Vin, Uout, Vout, FX, FY, coef, Vout == nullptr);
+  return tb2d_region<PERIODIC, true>(sh, nx, ny, k, kq, x0, y0, Uin, Vin, Uout, Vout, FX, FY, pf, pf, pin, pout, coef,
+                                     Vout == nullptr);
 }
 
 // FP32 items hold a 4 x 4 block of cells per thread in registers: two CTAs per SM
@@ -544,6 +547,7 @@ __global__ void __launch_bounds__(BT_THREADS, bt_min_blocks<S, A>()) k_batched(c
       const float* Vin = static_cast<const float*>(Vin_v);
       float* Uout = static_cast<float*>(Uout_v);
       float* Vout = static_cast<float*>(Vout_v);
+      const int pin = Uin_v == P.u ? P.nx : P.pitch, pout = Uout_v == P.u ? P.nx : P.pitch;
       bool bad = false;
       // the item's tiles: consecutive tiles of the pass, one region after another
       for (int g = 0; g < h.group; ++g) {
@@ -553,10 +557,10 @@ __global__ void __launch_bounds__(BT_THREADS, bt_min_blocks<S, A>()) k_batched(c
         const int x0 = tx_i * h.tx - h.k, y0 = ty_i * h.ty - h.k;
         bad |= periodic ? fp32_region_call<true>(rsh, P.nx, P.ny, h.k, kq, x0, y0, Uin, Vin, Uout, Vout,
                                                  static_cast<const float*>(P.fx), static_cast<const float*>(P.fy),
-                                                 P.coef + 2 * l0)
+                                                 P.fpitch, pin, pout, P.coef + 2 * l0)
                         : fp32_region_call<false>(rsh, P.nx, P.ny, h.k, kq, x0, y0, Uin, Vin, Uout, Vout,
                                                   static_cast<const float*>(P.fx), static_cast<const float*>(P.fy),
-                                                  P.coef + 2 * l0);
+                                                  P.fpitch, pin, pout, P.coef + 2 * l0);
         __syncthreads();  // the region's shared exchange buffers are reused by the next tile
       }
       if (bad) atomicOr(h.status, ST_NONFINITE);
@@ -747,6 +751,14 @@ frkc2_status batch_geometry(int nprob, const frkc2_plan_t* plans, const frkc2_pr
   return FRKC2_OK;
 }
 
+// faces of one problem: FP32 rows padded to a multiple of 4 (launch_faces_padded), else as launch_faces lays them
+size_t batch_fx_bytes(const BProb& P, bool padded, size_t AB) {
+  return align256(size_t(P.ny) * (padded ? P.fpitch : P.nx + 1) * AB);
+}
+size_t batch_fy_bytes(const BProb& P, bool padded, size_t AB) {
+  return align256(size_t(P.ny + 1) * (padded ? P.fpitch : P.nx) * AB);
+}
+
 frkc2_status batch_plan(int nprob, const frkc2_plan_t* plans, const frkc2_problem* probs, const double* dt,
                         const int* nsteps, const frkc2_tuning* tune, BatchPlanHost& B, int& k, int& tx, int& ty) {
   frkc2_status v = batch_geometry(nprob, plans, probs, nsteps, tune, &k, &tx, &ty);
@@ -772,6 +784,8 @@ frkc2_status batch_plan(int nprob, const frkc2_plan_t* plans, const frkc2_proble
     BProb& P = B.probs[r];
     P.nx = int(p.n[0]);
     P.ny = int(p.n[1]);
+    P.pitch = (P.nx + 3) / 4 * 4;
+    P.fpitch = (P.nx + 1 + 3) / 4 * 4;
     P.tiles_x = (P.nx + tx - 1) / tx;
     P.tiles_total = P.tiles_x * ((P.ny + ty - 1) / ty);
     P.ntiles = (P.tiles_total + group - 1) / group;
@@ -817,16 +831,16 @@ frkc2_status batch_plan(int nprob, const frkc2_plan_t* plans, const frkc2_proble
   B.counter_bytes = 16 + sizeof(unsigned) * size_t(nprob);
   off += align256(B.counter_bytes);
   B.off_faces = off;
-  const bool streaming = batch_streaming(probs[0].precision, k, tune);
+  const bool streaming = batch_streaming(probs[0].precision, k, tune), padded = probs[0].precision == FRKC2_FP32;
   for (int r = 0; r < nprob; ++r) {
     const BProb& P = B.probs[r];
-    off += align256(size_t(P.ny) * (P.nx + 1) * AB) + align256(size_t(P.ny + 1) * P.nx * AB);
+    off += batch_fx_bytes(P, padded, AB) + batch_fy_bytes(P, padded, AB);
     if (streaming) off += align256(size_t(P.ny + 1) * (P.nx + 1) * 2 * AB);  // face pairs
   }
   B.off_states = off;
   for (int r = 0; r < nprob; ++r) {
     const BProb& P = B.probs[r];
-    off += 4 * align256(size_t(P.nx) * P.ny * SB);
+    off += 4 * align256(size_t(padded ? P.pitch : P.nx) * P.ny * SB);
   }
   B.total = off;
   return FRKC2_OK;
@@ -889,16 +903,16 @@ frkc2_status frkc2_batch_prepare(int nprob, const frkc2_plan_t* plans, const frk
   char* base = static_cast<char*>(ws);
   const int prec = probs[0].precision;
   const size_t SB = state_bytes(prec), AB = arith_bytes(prec);
-  const bool streaming = batch_streaming(prec, k, tune);
+  const bool streaming = batch_streaming(prec, k, tune), padded = prec == FRKC2_FP32;
   // per-problem pointers and face conductivities
   size_t fo = B.off_faces, so = B.off_states;
   for (int r = 0; r < nprob; ++r) {
     BProb& P = B.probs[r];
     const int i = B.order[r];
     void* fx = base + fo;
-    fo += align256(size_t(P.ny) * (P.nx + 1) * AB);
+    fo += batch_fx_bytes(P, padded, AB);
     void* fy = base + fo;
-    fo += align256(size_t(P.ny + 1) * P.nx * AB);
+    fo += batch_fy_bytes(P, padded, AB);
     P.fx = fx;
     P.fy = fy;
     P.fen = nullptr;
@@ -907,7 +921,7 @@ frkc2_status frkc2_batch_prepare(int nprob, const frkc2_plan_t* plans, const frk
       fo += align256(size_t(P.ny + 1) * (P.nx + 1) * 2 * AB);
       P.fen = fen;
     }
-    const size_t sb = align256(size_t(P.nx) * P.ny * SB);
+    const size_t sb = align256(size_t(padded ? P.pitch : P.nx) * P.ny * SB);
     P.ua = base + so;
     P.va = base + so + sb;
     P.ub = base + so + 2 * sb;
@@ -915,7 +929,9 @@ frkc2_status frkc2_batch_prepare(int nprob, const frkc2_plan_t* plans, const frk
     so += 4 * sb;
     P.u = u[i];
     P.coef = reinterpret_cast<const double*>(base + B.off_coef) + B.coef_off[r];
-    if (launch_faces(probs[i], fx, fy, nullptr, st) != cudaSuccess) return FRKC2_ECUDA;
+    if ((padded ? launch_faces_padded(probs[i], static_cast<float*>(fx), static_cast<float*>(fy), P.fpitch, st)
+                : launch_faces(probs[i], fx, fy, nullptr, st)) != cudaSuccess)
+      return FRKC2_ECUDA;
     if (streaming && launch_face_pairs(probs[i], fx, fy, const_cast<void*>(P.fen), st) != cudaSuccess)
       return FRKC2_ECUDA;
   }

@@ -25,6 +25,8 @@
 // state of a shared-memory ping-pong.
 #pragma once
 
+#include <cstdint>
+
 #include <cuda_runtime.h>
 
 namespace frkc2 {
@@ -52,12 +54,14 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a
 // x0, y0: grid coordinates of the region's corner (tile origin - k).  coef(j, ca, cb) gives the
 // stage coefficients.  L1BYPASS: state loads through L2 only (buffers written by other CTAs
 // of the same launch).  Returns true if a stored value is not finite (when check_finite).
+// pfx, pfy, pin, pout: row pitches of the faces and of the state read and written.  A thread's rows move as
+// 16-byte vectors where pitch, k and pointer keep them aligned and they lie in the grid in one piece.
 template <bool PERIODIC, bool L1BYPASS, class Coef>
 __device__ __forceinline__ bool tb2d_region(RegionShared& sh, int nx, int ny, int k, int kq, int x0, int y0,
                                             const float* __restrict__ Uin, const float* __restrict__ Vin,
                                             float* __restrict__ Uo, float* __restrict__ Vo,
                                             const float* __restrict__ FX, const float* __restrict__ FY,
-                                            Coef coef, bool check_finite) {
+                                            int pfx, int pfy, int pin, int pout, Coef coef, bool check_finite) {
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 
   // wrapped (periodic) or raw (Dirichlet) grid rows / columns of the thread's cells; the fifth
@@ -72,51 +76,91 @@ __device__ __forceinline__ bool tb2d_region(RegionShared& sh, int nx, int ny, in
     xin[i] = gx >= 0 && gx < nx;
     yin[i] = gy >= 0 && gy < ny;
   }
-  // fx[r][c]: x face c of row r (the west face of cell c; c = 4 is the east face of cell 3);
-  // fy[r][c]: y face r of column c (the south face of row r; r = 4 is the north face of row 3)
-  float fx[4][5], fy[5][4];
   unsigned inside = 0;  // Dirichlet: bit 4r + c set if cell (r, c) lies in the grid
-#pragma unroll
-  for (int r = 0; r < 5; ++r) {
-#pragma unroll
-    for (int c = 0; c < 5; ++c) {
-      if (r < 4) {
-        float v = 0.f;
-        if (PERIODIC || (yin[r] && gxc[c] >= 0 && gxc[c] <= nx)) v = FX[size_t(gyr[r]) * (nx + 1) + gxc[c]];
-        fx[r][c] = v;
-      }
-      if (c < 4) {
-        float v = 0.f;
-        if (PERIODIC || (xin[c] && gyr[r] >= 0 && gyr[r] <= ny)) v = FY[size_t(gyr[r]) * nx + gxc[c]];
-        fy[r][c] = v;
-        if (r < 4 && xin[c] && yin[r]) inside |= 1u << (4 * r + c);
-      }
-    }
-  }
-  // the state as horizontal cell pairs: U2[r][h] = (U[r][2h], U[r][2h + 1]); the y faces too
-  float2 U2[4][2], V2[4][2], FY2[5][2];
-#pragma unroll
-  for (int r = 0; r < 5; ++r)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) FY2[r][h] = make_float2(fy[r][2 * h], fy[r][2 * h + 1]);
 #pragma unroll
   for (int r = 0; r < 4; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      float uu = 0.f, vv = 0.f;
-      if (PERIODIC || (inside & (1u << (4 * r + c)))) {
-        const size_t g = size_t(gyr[r]) * nx + gxc[c];
-        uu = L1BYPASS ? __ldcg(Uin + g) : Uin[g];
-        if (Vin) vv = L1BYPASS ? __ldcg(Vin + g) : Vin[g];
-      }
-      if (c & 1) {
-        U2[r][c >> 1].y = uu;
-        V2[r][c >> 1].y = vv;
-      } else {
-        U2[r][c >> 1].x = uu;
-        V2[r][c >> 1].x = vv;
+    for (int c = 0; c < 4; ++c)
+      if (xin[c] && yin[r]) inside |= 1u << (4 * r + c);
+  const bool run = (gxc[0] & 3) == 0 && gxc[3] == gxc[0] + 3 && (PERIODIC || (xin[0] && xin[3]));
+  // fx[r][c]: x face c of row r (the west face of cell c; c = 4 is the east face of cell 3);
+  // FY2[r]: y faces r as cell pairs (the south faces of row r; r = 4 the north faces of row 3)
+  float fx[4][5];
+  float2 FY2[5][2];
+  if (run && ((pfx | pfy) & 3) == 0) {
+#pragma unroll
+    for (int r = 0; r < 5; ++r) {
+      float4 y = make_float4(0.f, 0.f, 0.f, 0.f), x = y;
+      float x4 = 0.f;
+      if (PERIODIC || (gyr[r] >= 0 && gyr[r] <= ny)) y = *reinterpret_cast<const float4*>(FY + size_t(gyr[r]) * pfy + gxc[0]);
+      FY2[r][0] = make_float2(y.x, y.y);
+      FY2[r][1] = make_float2(y.z, y.w);
+      if (r < 4) {
+        if (PERIODIC || yin[r]) {
+          const float* q = FX + size_t(gyr[r]) * pfx + gxc[0];
+          x = *reinterpret_cast<const float4*>(q);
+          x4 = q[4];  // (periodic face nx repeats face 0)
+        }
+        fx[r][0] = x.x;
+        fx[r][1] = x.y;
+        fx[r][2] = x.z;
+        fx[r][3] = x.w;
+        fx[r][4] = x4;
       }
     }
+  } else {
+#pragma unroll
+    for (int r = 0; r < 5; ++r) {
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {
+        if (r < 4) {
+          float v = 0.f;
+          if (PERIODIC || (yin[r] && gxc[c] >= 0 && gxc[c] <= nx)) v = FX[size_t(gyr[r]) * pfx + gxc[c]];
+          fx[r][c] = v;
+        }
+        if (c < 4) {
+          float v = 0.f;
+          if (PERIODIC || (xin[c] && gyr[r] >= 0 && gyr[r] <= ny)) v = FY[size_t(gyr[r]) * pfy + gxc[c]];
+          (c & 1 ? FY2[r][c >> 1].y : FY2[r][c >> 1].x) = v;
+        }
+      }
+    }
+  }
+  // the state as horizontal cell pairs: U2[r][h] = (U[r][2h], U[r][2h + 1])
+  float2 U2[4][2], V2[4][2];
+  if (run && (pin & 3) == 0 && (reinterpret_cast<uintptr_t>(Uin) & 15) == 0) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      float4 u = make_float4(0.f, 0.f, 0.f, 0.f), v = u;
+      if (PERIODIC || yin[r]) {
+        const size_t g = size_t(gyr[r]) * pin + gxc[0];
+        const float4* qu = reinterpret_cast<const float4*>(Uin + g);
+        u = L1BYPASS ? __ldcg(qu) : *qu;
+        if (Vin) {
+          const float4* qv = reinterpret_cast<const float4*>(Vin + g);
+          v = L1BYPASS ? __ldcg(qv) : *qv;
+        }
+      }
+      U2[r][0] = make_float2(u.x, u.y);
+      U2[r][1] = make_float2(u.z, u.w);
+      V2[r][0] = make_float2(v.x, v.y);
+      V2[r][1] = make_float2(v.z, v.w);
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        float uu = 0.f, vv = 0.f;
+        if (PERIODIC || (inside & (1u << (4 * r + c)))) {
+          const size_t g = size_t(gyr[r]) * pin + gxc[c];
+          uu = L1BYPASS ? __ldcg(Uin + g) : Uin[g];
+          if (Vin) vv = L1BYPASS ? __ldcg(Vin + g) : Vin[g];
+        }
+        (c & 1 ? U2[r][c >> 1].y : U2[r][c >> 1].x) = uu;
+        (c & 1 ? V2[r][c >> 1].y : V2[r][c >> 1].x) = vv;
+      }
+  }
 
   const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int j = 0; j < kq; ++j) {
@@ -195,20 +239,29 @@ __device__ __forceinline__ bool tb2d_region(RegionShared& sh, int nx, int ny, in
 
   // store the output tile: region cells at distance >= k from the region edge
   bool bad = false;
+  const int gx0 = x0 + 4 * tx;
+  const bool vout = (pout & 3) == 0 && (reinterpret_cast<uintptr_t>(Uo) & 15) == 0 && (gx0 & 3) == 0 && 4 * tx >= k &&
+                    4 * tx + 4 <= RT_R - k && gx0 + 4 <= nx;
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     const int ry = 4 * ty + r;
     const int gy = y0 + ry;
     if (ry < k || ry >= RT_R - k || gy >= ny) continue;
+    const size_t row = size_t(gy) * pout;
+    if (vout) {
+      *reinterpret_cast<float4*>(Uo + row + gx0) = make_float4(U2[r][0].x, U2[r][0].y, U2[r][1].x, U2[r][1].y);
+      if (Vo) *reinterpret_cast<float4*>(Vo + row + gx0) = make_float4(V2[r][0].x, V2[r][0].y, V2[r][1].x, V2[r][1].y);
+    }
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const int rx = 4 * tx + c;
-      const int gx = x0 + rx;
+      const int gx = gx0 + c;
       if (rx < k || rx >= RT_R - k || gx >= nx) continue;
-      const size_t g = size_t(gy) * nx + gx;
       const float uu = (c & 1) ? U2[r][c >> 1].y : U2[r][c >> 1].x;
-      Uo[g] = uu;
-      if (Vo) Vo[g] = (c & 1) ? V2[r][c >> 1].y : V2[r][c >> 1].x;
+      if (!vout) {
+        Uo[row + gx] = uu;
+        if (Vo) Vo[row + gx] = (c & 1) ? V2[r][c >> 1].y : V2[r][c >> 1].x;
+      }
       if (check_finite) bad |= (__float_as_uint(uu) & 0x7f800000u) == 0x7f800000u;
     }
   }
