@@ -362,7 +362,7 @@ frkc2_status frkc2_adjoint_backward(frkc2_plan_t plan, const frkc2_problem* prob
  * counters and launches, so it can be captured in a CUDA graph and replayed.
  * Work items: FP32 and DFLOAT problems run register-tiled 64 x 64 regions of k stages (tile
  * 64 - 2k, default k = 8, the fastest on a mixed batch; DFLOAT with float-pair state),
- * tune->tile_z consecutive regions of one pass per item (default 4); FP64 / MIXED problems
+ * tune->tile_z consecutive regions of one pass per item (default 1 to 4 by the size of the batch); FP64 / MIXED problems
  * with k = 1 (the default), and DFLOAT with k = 1, run the single-stage streaming body on
  * tiles of 31 columns x tune->tile_y rows (default 128); FP64 / MIXED with k > 1 or kernel = 1
  * a k-stage shared-memory tile of tune->tile_x x tune->tile_y (DFLOAT: FRKC2_EUNSUPPORTED).

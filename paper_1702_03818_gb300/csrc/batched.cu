@@ -693,16 +693,26 @@ struct BatchPlanHost {
   size_t off_hdr, off_probs, off_round, off_cum, off_coef, off_counters, off_faces, off_states, total;
   size_t counter_bytes;
   int nrounds;
+  int group;  // regions per work item
   long long total_items;
 };
 
-// FP32 and DFLOAT region items: consecutive 64 x 64 regions of one pass per work item
-// (tune->tile_z; default 4),
-// which spreads the per-item hand-over (ticket, decode, dependency check, completion fence)
-// over several regions
-int batch_group(int precision, const frkc2_tuning* tune, bool streaming) {
+// FP32 and DFLOAT region items: consecutive 64 x 64 regions of one pass per work item (tune->tile_z), which
+// spreads the per-item hand-over (ticket, decode, dependency check, completion fence) over several regions.  The
+// default is up to 4, fewer where a round has too few regions to go round: one per item below 3 regions a
+// resident CTA, since an item's regions run one after another.  (FP32, k = 8, 1 / 2 / 4 regions an item: 32 problems
+// with 9.4 regions a CTA and round on average 3879 / 3439 / 3215 us, 12 with 3.2 663 / 619 / 777, 28 with 2.4
+// 1138 / 1177 / 1477, 9 with 0.2 237 / 379 / 617.)
+int batch_group(int precision, const frkc2_tuning* tune, bool streaming, double regions_per_round) {
   if (streaming || (precision != FRKC2_FP32 && precision != FRKC2_DFLOAT)) return 1;
-  return (tune && tune->tile_z) ? tune->tile_z : 4;
+  if (tune && tune->tile_z) return tune->tile_z;
+  static const int sms = [] {
+    int dev = 0, n = 152;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      n = 152;
+    return n;
+  }();
+  return std::max(1, std::min(4, int(regions_per_round / (1.5 * 2 * sms))));
 }
 
 // FP64 / MIXED batches with one stage per pass run streaming items unless kernel 1 (the shared-
@@ -764,13 +774,18 @@ frkc2_status batch_plan(int nprob, const frkc2_plan_t* plans, const frkc2_proble
   frkc2_status v = batch_geometry(nprob, plans, probs, nsteps, tune, &k, &tx, &ty);
   if (v != FRKC2_OK) return v;
   const size_t SB = state_bytes(probs[0].precision), AB = arith_bytes(probs[0].precision);
-  const int group = batch_group(probs[0].precision, tune, batch_streaming(probs[0].precision, k, tune));
-  if (group < 1 || group > 64) return FRKC2_EINVAL;
   std::vector<int> T(nprob);
+  double regions = 0.0;
+  int most = 1;
   for (int i = 0; i < nprob; ++i) {
     const int P = (plans[i]->s + k - 1) / k;
     T[i] = nsteps[i] * P;
+    most = std::max(most, T[i]);
+    regions += double((probs[i].n[0] + tx - 1) / tx) * double((probs[i].n[1] + ty - 1) / ty) * T[i];
   }
+  const int group = batch_group(probs[0].precision, tune, batch_streaming(probs[0].precision, k, tune), regions / most);
+  if (group < 1 || group > 64) return FRKC2_EINVAL;
+  B.group = group;
   B.order.resize(nprob);
   std::iota(B.order.begin(), B.order.end(), 0);
   std::stable_sort(B.order.begin(), B.order.end(), [&](int a, int b) { return T[a] > T[b]; });
@@ -943,7 +958,7 @@ frkc2_status frkc2_batch_prepare(int nprob, const frkc2_plan_t* plans, const frk
   h.ty = ty;
   h.k = k;
   h.stream_rows = streaming ? ty : 0;
-  h.group = batch_group(prec, tune, streaming);
+  h.group = B.group;
   h.fault_inject = tune ? tune->fault_inject : 0;
   h.total_items = B.total_items;
   h.wait_limit = (tune && tune->wait_limit > 0) ? tune->wait_limit : DEFAULT_WAIT_LIMIT;
