@@ -364,7 +364,7 @@ frkc2_status frkc2_adjoint_backward(frkc2_plan_t plan, const frkc2_problem* prob
  * 64 - 2k, default k = 8, the fastest on a mixed batch; DFLOAT with float-pair state),
  * tune->tile_z consecutive regions of one pass per item (default 1 to 4 by the size of the batch); FP64 / MIXED problems
  * with k = 1 (the default), and DFLOAT with k = 1, run the single-stage streaming body on
- * tiles of 31 columns x tune->tile_y rows (default 128); FP64 / MIXED with k > 1 or kernel = 1
+ * tiles of 31 columns x tune->tile_y rows (default 128, FP64 8 to 128); FP64 / MIXED with k > 1 or kernel = 1
  * a k-stage shared-memory tile of tune->tile_x x tune->tile_y (DFLOAT: FRKC2_EUNSUPPORTED).
  *   plans, probs, dt, nsteps, u : host arrays of nprob entries (u[i] device pointers).    */
 frkc2_status frkc2_batch_workspace_size(int nprob, const frkc2_plan_t* plans,

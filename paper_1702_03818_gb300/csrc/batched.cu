@@ -697,6 +697,17 @@ struct BatchPlanHost {
   long long total_items;
 };
 
+// SMs of the device (152 where it cannot be asked).
+int batch_sms() {
+  static const int sms = [] {
+    int dev = 0, n = 152;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      n = 152;
+    return n;
+  }();
+  return sms;
+}
+
 // FP32 and DFLOAT region items: consecutive 64 x 64 regions of one pass per work item (tune->tile_z), which
 // spreads the per-item hand-over (ticket, decode, dependency check, completion fence) over several regions.  The
 // default is up to 4, fewer where a round has too few regions to go round: one per item below 3 regions a
@@ -706,13 +717,7 @@ struct BatchPlanHost {
 int batch_group(int precision, const frkc2_tuning* tune, bool streaming, double regions_per_round) {
   if (streaming || (precision != FRKC2_FP32 && precision != FRKC2_DFLOAT)) return 1;
   if (tune && tune->tile_z) return tune->tile_z;
-  static const int sms = [] {
-    int dev = 0, n = 152;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      n = 152;
-    return n;
-  }();
-  return std::max(1, std::min(4, int(regions_per_round / (1.5 * 2 * sms))));
+  return std::max(1, std::min(4, int(regions_per_round / (1.5 * 2 * batch_sms()))));
 }
 
 // FP64 / MIXED batches with one stage per pass run streaming items unless kernel 1 (the shared-
@@ -727,6 +732,23 @@ size_t batch_smem(int precision, int tx, int ty, int k, bool streaming = false) 
   if (precision == FRKC2_FP32 || streaming) return 0;
   if (precision == FRKC2_DFLOAT) return sizeof(DfShared);  // the float-pair regions
   return size_t(tx + 2 * k) * (ty + 2 * k) * (4 * state_bytes(precision) + 2 * arith_bytes(precision));
+}
+
+// Rows of a streaming item, FP64: 8 to 128, a multiple of the CTA's 8 warps, so many that an average round has
+// about 1.15 items for each of two CTAs per SM; with fewer items SMs idle, with more the hand-overs count.  (6
+// problems of 200^2 to 500^2, rows 8 / 24 / 64 / 128: 3197 / 1937 / 2780 / 4855 us; 4 of 40^2 to 100^2 704 / 1010 / 1630 / 1587; 16 of
+// 200^2 to 512^2 21418 / 10549 / 7069 / 7215.)  MIXED keeps 128: where a block starts decides which products of its
+// float flux sums the two rows of an unrolled iteration share, and with that their rounding.
+int batch_stream_rows(int nprob, const frkc2_plan_t* plans, const frkc2_problem* probs, const int* nsteps) {
+  if (probs[0].precision != FRKC2_FP64) return 128;
+  double rows = 0.0, most = 1.0;  // (column chunk, row) pairs over all passes, and the longest chain of passes
+  for (int i = 0; i < nprob; ++i) {
+    const double passes = double(nsteps[i]) * plans[i]->s;
+    rows += double((probs[i].n[0] + BS_COLS - 1) / BS_COLS) * double(probs[i].n[1]) * passes;
+    most = std::max(most, passes);
+  }
+  const double r = rows / most / (1.15 * 2 * batch_sms());
+  return r >= 128.0 ? 128 : std::max(8, int(r / 8.0) * 8);
 }
 
 frkc2_status batch_geometry(int nprob, const frkc2_plan_t* plans, const frkc2_problem* probs, const int* nsteps,
@@ -752,7 +774,7 @@ frkc2_status batch_geometry(int nprob, const frkc2_plan_t* plans, const frkc2_pr
     tx = ty = RT_R - 2 * k;
   } else if (batch_streaming(p0.precision, k, tune)) {  // streaming items: 31 columns x a row block
     tx = BS_COLS;
-    ty = (tune && tune->tile_y) ? tune->tile_y : 128;
+    ty = (tune && tune->tile_y) ? tune->tile_y : batch_stream_rows(nprob, plans, probs, nsteps);
   }
   if (batch_smem(p0.precision, tx, ty, k, batch_streaming(p0.precision, k, tune)) > 200 * 1024) return FRKC2_EINVAL;
   *k_out = k;
