@@ -17,6 +17,9 @@
 // floating-point instructions per cell-stage, with no product contracted into an add, so every
 // launch shape gives the same bits.  At the end of each step the state is Re W^L.  The stage
 // coefficients of the whole plan (up to 1024 stages) are copied once to shared memory.
+//
+// In FP64 the library's own shapes put the two components of a cell on different lanes where that is faster
+// (k_small1d_split, the same bits).
 #include <algorithm>
 #include <memory>
 
@@ -204,7 +207,134 @@ __global__ void __launch_bounds__(S1_TMAX, 1) k_small1d(const Small1dArgs a) {
   if (bad) atomicOr(a.status, ST_NONFINITE);
 }
 
-template <class S, class A, bool PERIODIC, int R>
+// FP64 with the two components of a cell on different lanes: lanes 0 .. 15 of a warp hold U of 16 slots of R
+// cells, lanes 16 .. 31 V of the same.  The FP64 pipe of an SM sub-partition takes 64 clocks for a warp instruction
+// whatever its lanes do, and the job is bound by the chain of a stage, so what counts is the FP64 instructions a
+// warp issues per stage: 5 R here (difference, flux product, f, two updates; the partner's f comes by a shuffle)
+// against 10 R + 2 with both components on a lane, for twice the warps, which small jobs leave idle.  Slot 0 is a
+// ghost that holds the last cell of the warp before, so that every west flux product comes from the adjacent lane.
+// The operations of a cell are those of k_small1d in their order: the same bits.  N = 256 in 8 CTAs: 0.48 us a stage
+// against 0.64, of which the exchange between CTAs 0.03; the rest is the chain difference - product - shuffle - f -
+// shuffle - update behind one CTA barrier.
+template <bool PERIODIC, int R>
+__global__ void __launch_bounds__(S1_TMAX, 1) k_small1d_split(const Small1dArgs a) {
+  __shared__ double wlo[2][2][S1_WMAX];    // [parity][component]: each warp's first own cell
+  __shared__ double whi[2][2][S1_WMAX];    // its last
+  __shared__ double own_lo[2][2][S1_HMAX]; // the chunk's first H cells, by exchange parity and component
+  __shared__ double own_hi[2][2][S1_HMAX]; // its last H cells
+  __shared__ double cs[2][S1_MAXS];        // the stage coefficients (ca, cb)
+  cg::cluster_group cluster = cg::this_cluster();
+  const int CL = int(cluster.num_blocks());
+  const int c = int(cluster.block_rank());
+  const int t = threadIdx.x, nt = blockDim.x, lane = t & 31, wid = t >> 5, nw = nt >> 5;
+  const int comp = lane >> 4, slot = lane & 15;
+  const int n = a.n, H = a.H;
+  const int c0 = int((long long)c * n / CL), c1 = int((long long)(c + 1) * n / CL);
+  const int cp = (c + CL - 1) % CL, cn = (c + 1) % CL;
+  const int E = (c1 - c0) + 2 * H;               // cells of the extended chunk, from global c0 - H
+  const int lo = (wid * 15 + slot - 1) * R;      // the lane's first cell
+  const double* __restrict__ U0 = static_cast<const double*>(a.u);
+  const double* __restrict__ FX = static_cast<const double*>(a.fx);
+  auto wrapn = [n](int g) { return g < 0 ? g + n : (g >= n ? g - n : g); };  // |g| < 2n here
+
+  double X[R];           // the lane's component of its cells
+  double ke[R];          // the faces east of them
+  unsigned live = 0;     // bit i: cell i is updated (in the extended chunk and the grid, not a ghost)
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int e = lo + i, g = c0 - H + e;
+    const bool in = slot > 0 && e < E && (PERIODIC || (g >= 0 && g < n));
+    if (in) live |= 1u << i;
+    const int gi = PERIODIC ? wrapn(g) : g;
+    X[i] = in && comp == 0 && in_bounds(gi >= 0 && gi < n, a.status) ? U0[gi] : 0.0;
+    double v = 0.0;      // face g + 1 lies between cells g and g + 1
+    if (e >= -1 && e < E) {
+      const int fi = PERIODIC ? wrapn(g + 1) : g + 1;
+      if ((PERIODIC || (g + 1 >= 0 && g + 1 <= n)) && in_bounds(fi >= 0 && fi <= n, a.status)) v = FX[fi];
+    }
+    ke[i] = v;
+  }
+  for (int l = t; l < a.s; l += nt) {
+    cs[0][l] = a.ca[l];
+    cs[1][l] = a.cb[l];
+  }
+  cluster.sync();  // every CTA of the cluster is running before any remote access
+
+  bool bad = false;
+  int par = 0, xpar = 0, since = 0;  // stages since the last halo exchange (the halo starts exact)
+  for (int step = 0; step < a.nsteps; ++step) {
+    for (int l = 0; l < a.s; ++l, par ^= 1) {
+      if (H > 0 && since == H) {
+        // halo exchange: the chunk's own first and last H cells out, the neighbours' in
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          const int e = lo + i;
+          if (slot > 0 && e >= H && e < 2 * H && in_bounds(e - H < S1_HMAX, a.status)) own_lo[xpar][comp][e - H] = X[i];
+          if (slot > 0 && e >= E - 2 * H && e < E - H && in_bounds(e - (E - 2 * H) < S1_HMAX, a.status))
+            own_hi[xpar][comp][e - (E - 2 * H)] = X[i];
+        }
+        cluster.sync();
+        const double* rlo = cluster.map_shared_rank(&own_hi[xpar][comp][0], cp);  // global cells c0 - H .. c0 - 1
+        const double* rhi = cluster.map_shared_rank(&own_lo[xpar][comp][0], cn);  // global cells c1 .. c1 + H - 1
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          const int e = lo + i;
+          if (live & (1u << i)) {
+            if (e < H)
+              X[i] = rlo[e];
+            else if (e >= E - H)
+              X[i] = rhi[e - (E - H)];
+          }
+        }
+        xpar ^= 1;
+        since = 0;
+      }
+      // the ghost slot takes the last cell of the warp before, the last slot's east neighbour is the next
+      // warp's first cell; beyond the extended chunk's ends zero
+      double eX = __shfl_down_sync(0xffffffffu, X[0], 1, 16);
+      if (nw > 1) {
+        if (slot == 1) wlo[par][comp][wid] = X[0];
+        if (slot == 15) whi[par][comp][wid] = X[R - 1];
+        __syncthreads();
+        if (slot == 0) X[R - 1] = wid > 0 ? whi[par][comp][wid - 1] : 0.0;
+        if (slot == 15) eX = wid < nw - 1 ? wlo[par][comp][wid + 1] : 0.0;
+      } else if (slot == 15) {
+        eX = 0.0;
+      }
+      const double ca = cs[0][l], cb = comp ? cs[1][l] : -cs[1][l];
+      double x[R], P[R];
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        x[i] = (i + 1 < R ? X[i + 1 < R ? i + 1 : i] : eX) - X[i];
+        P[i] = mul_rn(ke[i], x[i]);
+      }
+      const double Pw = __shfl_up_sync(0xffffffffu, P[R - 1], 1, 16);
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        const double f = fma(ke[i], x[i], -(i > 0 ? P[i > 0 ? i - 1 : 0] : Pw));
+        const double fo = __shfl_xor_sync(0xffffffffu, f, 16);  // the other component's
+        if (live & (1u << i)) X[i] = fma(cb, fo, fma(ca, f, X[i]));
+      }
+      if (l == a.s - 1 && comp == 1) {  // step output: the real part
+#pragma unroll
+        for (int i = 0; i < R; ++i) X[i] = 0.0;
+      }
+      ++since;
+    }
+  }
+  cluster.sync();  // no CTA leaves while another may still read its shared memory
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int e = lo + i;
+    if (comp == 0 && slot > 0 && e >= H && e < E - H && in_bounds(c0 - H + e >= 0 && c0 - H + e < n, a.status)) {
+      static_cast<double*>(a.u)[c0 - H + e] = X[i];
+      bad |= bad1(X[i]);
+    }
+  }
+  if (bad) atomicOr(a.status, ST_NONFINITE);
+}
+
+template <class S, class A, bool PERIODIC, int R, bool SPLIT>
 cudaError_t launch_r(const Small1dArgs& a, int CL, int threads, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(CL, 1, 1);
@@ -218,18 +348,22 @@ cudaError_t launch_r(const Small1dArgs& a, int CL, int threads, cudaStream_t st)
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_small1d<S, A, PERIODIC, R>, a);
+  cudaError_t e;
+  if constexpr (SPLIT)
+    e = cudaLaunchKernelEx(&cfg, k_small1d_split<PERIODIC, R>, a);
+  else
+    e = cudaLaunchKernelEx(&cfg, k_small1d<S, A, PERIODIC, R>, a);
   count_launch();
   return e;
 }
 
-template <class S, class A, bool PERIODIC>
+template <class S, class A, bool PERIODIC, bool SPLIT = false>
 cudaError_t launch_t(const Small1dArgs& a, int CL, int threads, int R, cudaStream_t st) {
   switch (R) {
-    case 1: return launch_r<S, A, PERIODIC, 1>(a, CL, threads, st);
-    case 2: return launch_r<S, A, PERIODIC, 2>(a, CL, threads, st);
-    case 4: return launch_r<S, A, PERIODIC, 4>(a, CL, threads, st);
-    case 8: return launch_r<S, A, PERIODIC, 8>(a, CL, threads, st);
+    case 1: return launch_r<S, A, PERIODIC, 1, SPLIT>(a, CL, threads, st);
+    case 2: return launch_r<S, A, PERIODIC, 2, SPLIT>(a, CL, threads, st);
+    case 4: return launch_r<S, A, PERIODIC, 4, SPLIT>(a, CL, threads, st);
+    case 8: return launch_r<S, A, PERIODIC, 8, SPLIT>(a, CL, threads, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -247,8 +381,8 @@ cudaError_t launch_small1d(const frkc2_problem& p, const frkc2_plan_s& plan, dou
                            int threads_per_cta) {
   const int n = int(p.n[0]);
   const bool periodic = p.bc == FRKC2_BC_PERIODIC;
-  // cluster size (or the caller's): 32 cells a CTA, up to 8 CTAs (N = 256: FP64 0.89 ms a job
-  // against 1.22 in one CTA, FP32 0.16 against 0.20)
+  // cluster size (or the caller's): 32 cells a CTA, up to 8 CTAs (N = 256: FP64 0.64 us a stage
+  // on one lane a cell against 0.88 in one CTA, FP32 0.12 against 0.14)
   const bool f32 = p.precision == FRKC2_FP32;
   int CL = cluster > 0 ? std::min(S1_CMAX, std::min(cluster, n)) : std::max(1, std::min(S1_CMAX, n / 32));
   CL = std::max(CL, (n + S1_TMAX * S1_RMAX / 2 - 1) / (S1_TMAX * S1_RMAX / 2));  // room for a halo
@@ -274,6 +408,27 @@ cudaError_t launch_small1d(const frkc2_problem& p, const frkc2_plan_s& plan, dou
   int R = 1;
   while (R * threads < ext) R *= 2;
   if (R > S1_RMAX) return cudaErrorInvalidValue;
+  // FP64 in the library's own shape: components on separate lanes where that is the faster (us a stage, s = 32):
+  //   one cell a lane in up to 8 warps: ext 60 0.48 against 0.64, 90 0.58 / 0.65, 104 0.63 / 0.67; in 10 warps and
+  //   more (ext > 140) 0.79 / 0.80 and 1.05 / 0.97: both issue about the same FP64 work per cell there;
+  //   where one cell a thread doesn't hold the chunk: n = 4096 2.0 / 3.2, 6000 2.7 / 3.2 (the other form fills 512
+  //   threads with 2^i cells each, most of them beyond the chunk).
+  // The halo is the deepest (down to 8 stages per exchange) that needs the fewest warps: an exchange takes 0.35 us,
+  // a further warp 0.04 us a stage.
+  bool split = false;
+  if (p.precision == FRKC2_FP64 && cluster <= 0 && stages_per_exchange <= 0 && threads_per_cta <= 0) {
+    auto warps = [chunk](int h, int r) { return (chunk + 2 * h + 15 * r - 1) / (15 * r); };
+    const int hmin = std::min(H, 8);
+    int r = 1;
+    while (R > 1 && r < S1_RMAX && warps(hmin, r) > S1_WMAX) r *= 2;
+    const int w = warps(hmin, r);
+    if (w <= (R > 1 ? S1_WMAX : 8)) {
+      split = true;
+      R = r;
+      threads = 32 * w;
+      while (H > hmin && warps(H, r) > w) --H;
+    }
+  }
   auto a = std::make_unique<Small1dArgs>();
   a->u = u;
   a->fx = fx;
@@ -289,6 +444,9 @@ cudaError_t launch_small1d(const frkc2_problem& p, const frkc2_plan_s& plan, dou
   }
   switch (p.precision) {
     case FRKC2_FP64:
+      if (split)
+        return periodic ? launch_t<double, double, true, true>(*a, CL, threads, R, st)
+                        : launch_t<double, double, false, true>(*a, CL, threads, R, st);
       return periodic ? launch_t<double, double, true>(*a, CL, threads, R, st)
                       : launch_t<double, double, false>(*a, CL, threads, R, st);
     case FRKC2_FP32:
