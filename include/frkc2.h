@@ -105,7 +105,8 @@ typedef struct {
                         rows per CTA, 0 = one wave of CTAs)                                  */
   int tile_y;
   int tile_z;
-  int kernel;        /* 0 = library choice, 1 = generic shared-memory tile kernel,
+  int kernel;        /* 0 = library choice (FP64 2D with fixed conductivity and k = 0: up to
+                        about 550^2 the whole job in one cooperative launch), 1 = generic shared-memory tile kernel,
                         2 = 2D streaming kernel (k = 1 only), 3 = 2D FP32 temporally blocked
                         kernel, 4 = 2D real pair kernel (PAIRED plans only), 5 = 3D kernel
                         streaming along z (k = 1 only), 6 = 1D whole-job cluster kernel
@@ -114,11 +115,12 @@ typedef struct {
                         stage levels in flight, rows staged in shared memory by TMA bulk
                         copies (n[0] a multiple of 4 and >= 256, u 16-byte aligned, every
                         pass of 1, 2, 4, 6, 8, 10 or 12 stages; the FP32 2D default there)  */
-  long long wait_limit; /* batched launch and kernel 7 (its waits on the TMA row copies):
+  long long wait_limit; /* batched launch, FP64 2D whole job and kernel 7 (its waits on the TMA row copies):
                         polls a device wait makes before it gives up and latches
                         FRKC2_ETIMEOUT (0 = library default, 2^22 polls)                    */
   int fault_inject;  /* testing only: 1 = in the batched launch the first dependent work
-                        item waits on a counter nothing advances; in kernel 7 (passes of
+                        item waits on a counter nothing advances; in the FP64 2D whole job
+                        the first wait is for a stage nothing publishes; in kernel 7 (passes of
                         k = 8) the first pass leaves one row uncopied; either wait must run out */
 } frkc2_tuning;
 

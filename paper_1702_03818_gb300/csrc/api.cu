@@ -308,6 +308,11 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
     const cudaError_t e = launch_small1d(p, *plan, dt, nsteps, u, base + L.fx, a.status, st, cl, kx, th);
     return e == cudaSuccess ? FRKC2_OK : e == cudaErrorInvalidValue ? FRKC2_EINVAL : FRKC2_ECUDA;
   }
+  if (use_stream2d && kern == 0 && !(tune && tune->k) && resident2d_wins(p, s, nsteps, L.total - L.fen)) {
+    const cudaError_t e = launch_resident2d(p, *plan, dt, nsteps, u, base + L.fx, base + L.fy, base + L.fen, L.total - L.fen,
+                                            a.status, tune ? tune->wait_limit : 0, tune ? tune->fault_inject : 0, st);
+    return e == cudaSuccess ? FRKC2_OK : FRKC2_ECUDA;
+  }
   const void* curU = u;
   const void* curV = nullptr;
   if (use_paired) {

@@ -150,6 +150,12 @@ cudaError_t launch_pass_wf2d(const frkc2_problem& p, const PassArgs& a, const vo
 cudaError_t launch_small1d(const frkc2_problem& p, const frkc2_plan_s& plan, double dt, int nsteps, void* u,
                            const void* fx, unsigned* status, cudaStream_t st, int cluster, int stages_per_exchange,
                            int threads_per_cta);
+// FP64 2D whole job in one cooperative launch (pass_resident2d.cu): whether it is the choice for the problem, given
+// the room for packets; and the launch (packets: 256-byte aligned, zeroed by the call)
+bool resident2d_wins(const frkc2_problem& p, int s, int nsteps, size_t packet_bytes);
+cudaError_t launch_resident2d(const frkc2_problem& p, const frkc2_plan_s& plan, double dt, int nsteps, void* u, const void* fx,
+                              const void* fy, void* packets, size_t packet_bytes, unsigned* status, long long wait_limit,
+                              int fault_inject, cudaStream_t st);
 int stream3d_chunks(long long blocks, int nz, long long slots);
 bool stream3d_supported(const frkc2_problem& p);
 cudaError_t launch_pass_stream3d_f32(const frkc2_problem& p, const PassArgs& a, cudaStream_t st);
