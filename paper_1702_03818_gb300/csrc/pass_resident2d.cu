@@ -7,13 +7,13 @@
 // whatever its lanes do, so half-warp columns spread a grid more evenly over the 4 x SMs sub-partitions: 256^2 is
 // 1216 units of 3 or 4 rows, 34 FP64 instructions a stage for each and 2 units a sub-partition).  A CTA is cw x rh
 // neighbouring units, at most one CTA an SM.  256^2: 5.9 us a stage as one launch each at the full grid, 4.7 with the
-// launches spread over the SMs, 3.1 here: 2.1 of FP64 issue and about 0.9 for the edges' trip through L2.
+// launches spread over the SMs, 3.0 here: 2.1 of FP64 issue and about 0.9 for the edges' trip through L2.
 // Per stage a warp publishes its four edges, forms the differences inside the unit, takes its neighbours' edges and
 // updates its cells (a cell's operations and their order are those of the streaming pass, whose unrolled rows the
 // compiler contracts in either of two ways: the same bits or 4e-15 apart).  Edges go to
 // warps of the same CTA through shared memory, at one CTA barrier a stage, and to other CTAs as 16-byte packets,
 // two 64-bit words that hold half a value and the stage number each: a reader that sees the number has the
-// value, so there is no fence, flag or second trip through L2.  A slot is written again two stages on; by then the
+// value (resident2d.cuh), so there is no fence, flag or second trip through L2.  A slot is written again two stages on; by then the
 // writer has read the neighbour's edge of the stage between, which the neighbour published after reading the
 // slot.  Every wait is bounded: when it runs out the warp latches the time-out status and goes on without
 // waiting, so the launch ends.
@@ -23,6 +23,7 @@
 #include <cuda_runtime.h>
 
 #include "frkc2_internal.h"
+#include "resident2d.cuh"
 
 namespace frkc2 {
 namespace {
@@ -46,22 +47,8 @@ struct Resident2dArgs {
   double cb[RS_MAXS];   // dt Im a_l / dx^2
 };
 
-enum { SIDE_N = 0, SIDE_S = 1, SIDE_E = 2, SIDE_W = 3 };
-enum { EDGE_NONE = 0, EDGE_LOCAL = 1, EDGE_REMOTE = 2 };
-
 // packets of a CTA: [parity][N: cw x 32, S: cw x 32, E: rh x 2R, W: rh x 2R]
 __host__ __device__ inline int packet_half(int cw, int rh, int R) { return 64 * cw + 4 * R * rh; }
-
-__device__ __forceinline__ void put_packet(ulonglong2* p, double v, unsigned seq) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v), q = (unsigned long long)seq << 32;
-  asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(q | (b & 0xffffffffull)), "l"(q | (b >> 32)) : "memory");
-}
-__device__ __forceinline__ bool get_packet(const ulonglong2* p, double& v, unsigned seq) {
-  unsigned long long lo, hi;
-  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "l"(p) : "memory");
-  v = __longlong_as_double((long long)((hi << 32) | (lo & 0xffffffffull)));
-  return unsigned(lo >> 32) == seq && unsigned(hi >> 32) == seq;
-}
 
 template <int R>
 __global__ void __launch_bounds__(32 * RS_WMAX, 1) k_resident2d(const Resident2dArgs a) {
@@ -191,7 +178,7 @@ __global__ void __launch_bounds__(32 * RS_WMAX, 1) k_resident2d(const Resident2d
       const double dWe = xw - h[SIDE_W];
       const double dTop = h[SIDE_N] - top;
       double dS = X[0] - h[SIDE_S];
-      const double ca = a.ca[l], cb = comp ? a.cb[l] : -a.cb[l];
+      const double ca = a.ca[l], cb = flip(a.cb[l], comp == 0);
       const bool last = l == a.s - 1;
       double ks = kS;
 #pragma unroll
@@ -245,24 +232,9 @@ ResidentShape resident_shape(int nx, int ny, int sms, size_t bytes) {
       if (R > RS_RMAX) continue;
       if (size_t(nstrip) * nband * 2 * packet_half(cw, rh, R) * sizeof(ulonglong2) > bytes) continue;
       const double us = 0.56 + (0.027 * std::max(1.5, double((nw + 3) / 4)) + 0.015) * (8 * R + 2) + 0.03 * nw;
-      if (!best.R || us < best.us) best = {cw, rh, nstrip, nband, R, us};
+      if (!best.R || us <= best.us) best = {cw, rh, nstrip, nband, R, us};
     }
   return best;
-}
-
-struct DeviceInfo {
-  int sms, coop;
-};
-DeviceInfo device_info() {
-  static const DeviceInfo d = [] {
-    DeviceInfo v{0, 0};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&v.coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess)
-      v.sms = v.coop = 0;
-    return v;
-  }();
-  return d;
 }
 
 template <int R>
@@ -284,14 +256,14 @@ bool resident2d_wins(const frkc2_problem& p, int s, int nsteps, size_t packet_by
   if (p.ndim != 2 || p.precision != FRKC2_FP64 || p.kappa_kind == FRKC2_KAPPA_POWER || s > RS_MAXS) return false;
   if ((long long)nsteps * s < 4) return false;
   if ((long long)nsteps * s >= 0x7fffffffll || p.n[0] * p.n[1] > (1 << 20)) return false;
-  const DeviceInfo d = device_info();
+  const CoopDevice d = coop_device();
   return d.coop && resident_shape(int(p.n[0]), int(p.n[1]), d.sms, packet_bytes).R > 0;
 }
 
 cudaError_t launch_resident2d(const frkc2_problem& p, const frkc2_plan_s& plan, double dt, int nsteps, void* u, const void* fx,
                               const void* fy, void* packets, size_t packet_bytes, unsigned* status, long long wait_limit,
                               int fault_inject, cudaStream_t st) {
-  const ResidentShape sh = resident_shape(int(p.n[0]), int(p.n[1]), device_info().sms, packet_bytes);
+  const ResidentShape sh = resident_shape(int(p.n[0]), int(p.n[1]), coop_device().sms, packet_bytes);
   if (!sh.R) return cudaErrorInvalidValue;
   const size_t used = size_t(sh.nstrip) * sh.nband * 2 * packet_half(sh.cw, sh.rh, sh.R) * sizeof(ulonglong2);
   const cudaError_t e = cudaMemsetAsync(packets, 0, used, st);

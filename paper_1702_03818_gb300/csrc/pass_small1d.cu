@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(S1_TMAX, 1) k_small1d(const Small1dArgs a) {
 // warp issues per stage: 5 R here (difference, flux product, f, two updates; the partner's f comes by a shuffle)
 // against 10 R + 2 with both components on a lane, for twice the warps, which small jobs leave idle.  Slot 0 is a
 // ghost that holds the last cell of the warp before, so that every west flux product comes from the adjacent lane.
-// The operations of a cell are those of k_small1d in their order: the same bits.  N = 256 in 8 CTAs: 0.48 us a stage
+// The operations of a cell are those of k_small1d in their order: the same bits.  N = 256 in 8 CTAs: 0.45 us a stage
 // against 0.64, of which the exchange between CTAs 0.03; the rest is the chain difference - product - shuffle - f -
 // shuffle - update behind one CTA barrier.
 template <bool PERIODIC, int R>
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(S1_TMAX, 1) k_small1d_split(const Small1dArgs 
   __shared__ double whi[2][2][S1_WMAX];    // its last
   __shared__ double own_lo[2][2][S1_HMAX]; // the chunk's first H cells, by exchange parity and component
   __shared__ double own_hi[2][2][S1_HMAX]; // its last H cells
-  __shared__ double cs[2][S1_MAXS];        // the stage coefficients (ca, cb)
+  __shared__ double cs[3][S1_MAXS];        // the stage coefficients (ca, -cb, cb; a negation takes an FP64 slot)
   cg::cluster_group cluster = cg::this_cluster();
   const int CL = int(cluster.num_blocks());
   const int c = int(cluster.block_rank());
@@ -256,7 +256,8 @@ __global__ void __launch_bounds__(S1_TMAX, 1) k_small1d_split(const Small1dArgs 
   }
   for (int l = t; l < a.s; l += nt) {
     cs[0][l] = a.ca[l];
-    cs[1][l] = a.cb[l];
+    cs[1][l] = -a.cb[l];
+    cs[2][l] = a.cb[l];
   }
   cluster.sync();  // every CTA of the cluster is running before any remote access
 
@@ -301,7 +302,7 @@ __global__ void __launch_bounds__(S1_TMAX, 1) k_small1d_split(const Small1dArgs 
       } else if (slot == 15) {
         eX = 0.0;
       }
-      const double ca = cs[0][l], cb = comp ? cs[1][l] : -cs[1][l];
+      const double ca = cs[0][l], cb = cs[1 + comp][l];
       double x[R], P[R];
 #pragma unroll
       for (int i = 0; i < R; ++i) {
