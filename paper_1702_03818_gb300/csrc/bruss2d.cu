@@ -9,8 +9,9 @@
 // Re w, Im w), ping-ponged between two copies; the first stage of a step reads the caller's
 // real (v, w) and the last stage writes the real parts back there.
 //
-// Launch forms (FP32's default is a third one, k stages per pass in registers: bruss_tb2d.cu):
-//  * persistent (the FP64 default): ONE cooperative launch runs every stage of every step; the CTAs
+// Launch forms (FP32's default is another one, k stages per pass in registers: bruss_tb2d.cu; and that of FP64 on
+// small grids, the whole job in registers: bruss_resident2d.cu):
+//  * persistent (the default of larger FP64 grids): ONE cooperative launch runs every stage of every step; the CTAs
 //    are all co-resident (a multiple of the SM count).  Between stages a CTA waits only for
 //    the CTAs whose cells its stencil reads (the owners of the cells within one grid row of
 //    its own range, a handful), which are also the CTAs that read its cells: each CTA
@@ -550,6 +551,15 @@ frkc2_status frkc2_bruss_step(frkc2_plan_t plan, const frkc2_bruss_problem* prob
       const cudaError_t te = launch_bruss_tb2d(*prob, *plan, dt, nsteps, k, static_cast<float*>(v), static_cast<float*>(w), P,
                                                reinterpret_cast<unsigned*>(wsb + L.status), st);
       return te == cudaSuccess ? FRKC2_OK : FRKC2_ECUDA;
+    }
+  }
+  if (kern == 0) {  // FP64 grids that fit the SMs' registers (200^2, s = 16, 42 steps 3900 -> 3020 us)
+    const BrLayout L = br_layout(*prob);
+    if (bruss_resident_wins(*prob, plan->s, nsteps, L.total - L.flags)) {
+      const cudaError_t re = launch_bruss_resident(*prob, *plan, dt, nsteps, static_cast<double*>(v), static_cast<double*>(w),
+                                                   wsb + L.flags, L.total - L.flags, reinterpret_cast<unsigned*>(wsb + L.status),
+                                                   wait_limit, fault, st);
+      return re == cudaSuccess ? FRKC2_OK : FRKC2_ECUDA;
     }
   }
   const bool per = prob->bc == FRKC2_BC_PERIODIC;

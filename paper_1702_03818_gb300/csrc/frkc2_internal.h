@@ -156,6 +156,11 @@ bool resident2d_wins(const frkc2_problem& p, int s, int nsteps, size_t packet_by
 cudaError_t launch_resident2d(const frkc2_problem& p, const frkc2_plan_s& plan, double dt, int nsteps, void* u, const void* fx,
                               const void* fy, void* packets, size_t packet_bytes, unsigned* status, long long wait_limit,
                               int fault_inject, cudaStream_t st);
+// the same for the Brusselator in FP64 (bruss_resident2d.cu)
+bool bruss_resident_wins(const frkc2_bruss_problem& p, int s, int nsteps, size_t packet_bytes);
+cudaError_t launch_bruss_resident(const frkc2_bruss_problem& p, const frkc2_plan_s& plan, double dt, int nsteps, double* v, double* w,
+                                  void* packets, size_t packet_bytes, unsigned* status, long long wait_limit, int fault_inject,
+                                  cudaStream_t st);
 int stream3d_chunks(long long blocks, int nz, long long slots);
 bool stream3d_supported(const frkc2_problem& p);
 cudaError_t launch_pass_stream3d_f32(const frkc2_problem& p, const PassArgs& a, cudaStream_t st);
