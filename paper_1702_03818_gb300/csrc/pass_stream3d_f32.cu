@@ -9,8 +9,8 @@
 // scalar instructions.  A packed negation is not free, so the complex products take one difference in both signs.
 // The plane loop is unrolled by three with the roles of the three planes held rotated (no register
 // moves), and the passes between a step's first and last are instantiated for interleaved state.
-// 256^3, kappa(u), s = 32: 125 -> 86 us a pass (40 us at the copy bandwidth; 90 instructions a computed
-// cell against 239 an output cell before, at 55 % issue).
+// 256^3, kappa(u), s = 32: 125 -> 79 us a pass (40 us at the copy bandwidth; 90 instructions a computed
+// cell against 239 an output cell before, at 62 % issue).
 #include <algorithm>
 
 #include <cuda_runtime.h>
@@ -26,6 +26,13 @@ constexpr int F3_OX = 30;     // output columns per CTA
 // outweighs their halo rows: 256^3, s = 32, kappa(u), a pass (rows, warps, CTAs): (4, 4, 4) 85.7 us, (2, 8, 3)
 // 86.9, (2, 12, 2) 88.6, (4, 8, 2) 93.4, (4, 4, 5) 95.2, (2, 8, 4) 97.8.
 constexpr int F3_RY = 4, F3_MAXW = 4, F3_CTAS = 4;
+// Planes by which the prefetch into L2 (one instruction of a warp a plane) runs ahead of the load: from DRAM a load
+// took longer than the plane of work between it and its use (36 % of the warps' time).  256^3, s = 32, kappa(u), a step:
+// none 2750 us, 1 2568, 2 2542, 3 2550, 5 2570.  Only where the two states and the conductivities don't stay in L2
+// anyway, above F3_L2 bytes (s = 16, 2 steps, without / with: 160^3, 66 MB 753 / 770, with a field, 82 MB 626 / 647;
+// 176^3, 87 MB 989 / 987, field 928 / 894; 224^3 1975 / 1859, field 1789 / 1572).
+constexpr size_t F3_L2 = 86000000;
+constexpr int F3_AHEAD = 2;
 constexpr int F3_H = F3_RY / 2;  // a thread's pairs of rows
 constexpr int K3_FIELD = 0, K3_POWER = 1, K3_P25 = 2;  // as in pass_stream3d.cu
 
@@ -36,6 +43,7 @@ struct F3Args {
   int chunks;               // chunks along z
   int in_real, out_real;    // the pass reads / writes the real state instead of interleaved (U, V)
   int check_finite;
+  int prefetch;             // prefetch planes into L2
   const void* in;
   void* out;
   const float* kappa;       // FIELD: cell conductivities; nullptr: the constant kc
@@ -154,6 +162,22 @@ __global__ void __launch_bounds__(32 * F3_MAXW, F3_CTAS) k_stream3d_f32(const F3
       if (out_x && R >= 1 && R <= p.oy && gy < ny) outm |= 1u << r;
     }
     auto zin = [&](int z) -> unsigned { return PERIODIC || (z >= 0 && z < nz) ? inside : 0u; };
+    // the lane's 32 bytes of the warp's four rows in a plane, for the prefetch into L2
+    unsigned poff;
+    {
+      const int gy = gy0 + (lane >> 3), px = gx - lane + 4 * (lane & 7);
+      poff = (unsigned(PERIODIC ? wrapf3(gy, ny) : min(max(gy, 0), ny - 1)) * unsigned(nx) +
+              unsigned(PERIODIC ? wrapf3(px, nx) : min(max(px, 0), nx - 1))) * 8u;
+    }
+    auto prefetch = [&](int z) {
+      const char* base = static_cast<const char*>(p.in) + size_t(PERIODIC ? wrapf3(z, nz) : min(max(z, 0), nz - 1)) * plane * 8;
+      if (in_bounds(poff / 8 < plane, p.status)) {
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(base + poff));
+        if (!POWER && p.kappa && (lane & 1) == 0)
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(p.kappa) +
+                                                        (base - static_cast<const char*>(p.in)) / 2 + poff / 2));
+      }
+    };
     // W (and FIELD / CONST conductivities) of plane z; the offsets are 32-bit against a uniform base
     auto load = [&](int z, Plane3& q) {
       const size_t zo = size_t(PERIODIC ? wrapf3(z, nz) : min(max(z, 0), nz - 1)) * plane;
@@ -289,6 +313,7 @@ __global__ void __launch_bounds__(32 * F3_MAXW, F3_CTAS) k_stream3d_f32(const F3
       }
       Ft = topflux(u, Nn);
       if (z + 3 <= z1) load(z + 3, c);
+      if (CC && p.prefetch && z + 3 + F3_AHEAD <= z1) prefetch(z + 3 + F3_AHEAD);
       kap(l, zin(z + 2));
     };
     for (int z = z0; z < z1; z += 3) {
@@ -375,6 +400,7 @@ cudaError_t launch_pass_stream3d_f32(const frkc2_problem& p, const PassArgs& a, 
   s.kp = float(a.kp);
   s.ca = float(0.5 * a.ca[0]);
   s.cb = float(0.5 * a.cb[0]);
+  s.prefetch = size_t(a.nx) * a.ny * a.nz * (s.kappa ? 20 : 16) > F3_L2;
   s.status = a.status;
   const bool per = p.bc == FRKC2_BC_PERIODIC;
   if (p.kappa_kind != FRKC2_KAPPA_POWER) return launch_k<K3_FIELD>(s, per, st);
