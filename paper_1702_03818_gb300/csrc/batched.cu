@@ -26,6 +26,7 @@
 // with k > 1 (or kernel 1) they run a k-stage shared-memory tile pass.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <mutex>
 #include <numeric>
 #include <type_traits>
@@ -61,7 +62,7 @@ struct BProb {
   void* va;
   void* ub;
   void* vb;
-  const double* coef;  // (ca, cb) per stage, dt a_l / dx^2
+  const double* coef;  // (ca, cb) per stage, dt a_l / dx^2: two doubles, or for a float state two floats and padding (stage_coef)
   int pitch, fpitch;   // FP32 regions: rows of the workspace state and of the faces, padded to a multiple of 4
 };
 
@@ -229,7 +230,7 @@ __device__ __forceinline__ bool stream_item(const BProb& P, int cw, int r0, int 
       const size_t g = size_t(y) * nx + x;
       if (out_real) {
         Uo[g] = un;
-        bad |= !isfinite(double(un));
+        bad |= !isfinite(un);
       } else {
         S2 w;
         w.x = un;
@@ -384,6 +385,21 @@ __device__ __forceinline__ bool stream_item_df(const BProb& P, int cw, int r0, i
   return bad;
 }
 
+// The coefficients of stage j, in a float state's case rounded by the host: a conversion here takes the FP64 pipe of a
+// sub-partition for 64 clocks, and two of them a warp and stage were 19 % of a FP32 batch (32 problems of 64^2 to
+// 1024^2, 2 steps each: 3212 -> 3070 us).
+template <class S>
+__device__ __forceinline__ void stage_coef(const double* cf, int j, S& ca, S& cb) {
+  if constexpr (std::is_same<S, double>::value) {
+    ca = cf[2 * j];
+    cb = cf[2 * j + 1];
+  } else {
+    const float2 c = reinterpret_cast<const float2*>(cf)[2 * j];
+    ca = c.x;
+    cb = c.y;
+  }
+}
+
 // One DFLOAT region as a call of its own (not inlined), so that each of its variants gets the
 // register budget it has in the single-problem pass instead of sharing one with the item loop.
 template <bool PERIODIC, bool IN_REAL, bool OUT_REAL>
@@ -391,8 +407,7 @@ __device__ __noinline__ bool df_region_call(DfShared& sh, int nx, int ny, int k,
                                             const void* in, void* out, const float* FX, const float* FY,
                                             const double* cf) {
   auto coef = [&](int j, float& ca, float& cb) {
-    ca = float(cf[2 * j]);
-    cb = float(cf[2 * j + 1]);
+    stage_coef(cf, j, ca, cb);
   };
   return tb2d_df_region<PERIODIC, IN_REAL, OUT_REAL, true, false>(sh, nx, ny, k, kq, x0, y0, in, out, FX, FY, coef, true,
                                                           [] {});
@@ -405,8 +420,7 @@ __device__ __noinline__ bool fp32_region_call(RegionShared& sh, int nx, int ny, 
                                               const float* FX, const float* FY, int pf, int pin, int pout,
                                               const double* cf) {
   auto coef = [&](int j, float& ca, float& cb) {
-    ca = float(cf[2 * j]);
-    cb = float(cf[2 * j + 1]);
+    stage_coef(cf, j, ca, cb);
   };
   return tb2d_region<PERIODIC, true>(sh, nx, ny, k, kq, x0, y0, Uin, Vin, Uout, Vout, FX, FY, pf, pf, pin, pout, coef,
                                      Vout == nullptr);
@@ -519,7 +533,8 @@ __global__ void __launch_bounds__(BT_THREADS, bt_min_blocks<S, A>()) k_batched(c
       const int q = s_round < P.total_passes ? s_round % P.passes_per_step : 0;
       const bool in_real = q == 0, out_real = q == P.passes_per_step - 1;
       bool bad = false;
-      const float ca = float(P.coef[2 * l0]), cb = float(P.coef[2 * l0 + 1]);
+      float ca, cb;
+      stage_coef(P.coef, l0, ca, cb);
       const int r0 = tyi * h.stream_rows, r1 = min(r0 + h.stream_rows, P.ny);
       if (periodic) {
         if (in_real && out_real)
@@ -567,7 +582,8 @@ __global__ void __launch_bounds__(BT_THREADS, bt_min_blocks<S, A>()) k_batched(c
     } else if (h.stream_rows > 0) {
       // one stage: real input at a step's first stage, real output at its last
       const int q = s_round < P.total_passes ? s_round % P.passes_per_step : 0;
-      const S ca = S(P.coef[2 * l0]), cb = S(P.coef[2 * l0 + 1]);
+      S ca, cb;
+      stage_coef(P.coef, l0, ca, cb);
       const int r0 = tyi * h.stream_rows, r1 = min(r0 + h.stream_rows, P.ny);
       const bool in_real = q == 0, out_real = q == P.passes_per_step - 1;
       const bool bad = periodic ? stream_item<S, A, true>(P, txi, r0, r1, Uin_v, in_real, Uout_v, out_real, ca, cb)
@@ -622,7 +638,8 @@ __global__ void __launch_bounds__(BT_THREADS, bt_min_blocks<S, A>()) k_batched(c
         const S* vs = (j & 1) ? vb0 : vb1;
         S* ud = (j & 1) ? ub1 : ub0;
         S* vd = (j & 1) ? vb1 : vb0;
-        const S ca = S(P.coef[2 * (l0 + j - 1)]), cb = S(P.coef[2 * (l0 + j - 1) + 1]);
+        S ca, cb;
+        stage_coef(P.coef, l0 + j - 1, ca, cb);
         const int w = RX - 2 * j, hgt = RY - 2 * j;
         for (int idx = tid; idx < w * hgt; idx += BT_THREADS) {
           const int y = j + idx / w, x = j + idx % w;
@@ -660,7 +677,7 @@ __global__ void __launch_bounds__(BT_THREADS, bt_min_blocks<S, A>()) k_batched(c
         const S uu = uf[i];
         Uout[g] = uu;
         if (Vout) Vout[g] = vf[i];
-        if (!Vout && !isfinite(double(uu))) bad = true;
+        if (!Vout && !isfinite(uu)) bad = true;
       }
       if (bad) atomicOr(h.status, ST_NONFINITE);
     }
@@ -836,8 +853,13 @@ frkc2_status batch_plan(int nprob, const frkc2_plan_t* plans, const frkc2_proble
     if (dt) {
       if (!(dt[i] > 0.0) || !std::isfinite(dt[i])) return FRKC2_EINVAL;
       for (int l = 0; l < P.s; ++l) {
-        B.coef.push_back(dt[i] * plans[i]->a_re[l] / h2);
-        B.coef.push_back(dt[i] * plans[i]->a_im[l] / h2);
+        double c[2] = {dt[i] * plans[i]->a_re[l] / h2, dt[i] * plans[i]->a_im[l] / h2};
+        if (p.precision == FRKC2_FP32 || p.precision == FRKC2_DFLOAT) {
+          const float f[2] = {float(c[0]), float(c[1])};
+          std::memcpy(&c[0], f, sizeof f);
+        }
+        B.coef.push_back(c[0]);
+        B.coef.push_back(c[1]);
       }
     } else {
       B.coef.resize(B.coef.size() + 2 * size_t(P.s), 0.0);

@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(GEN_THREADS) k_pass_generic(const PassArgs p) 
       Uout[g] = uu;
       if (Vout) Vout[g] = vf[i];
       if (hat) static_cast<S*>(p.H_out)[g] = hb[i];
-      if (p.check_finite && !isfinite(double(uu))) bad = true;
+      if (p.check_finite && !isfinite(uu)) bad = true;
     }
   if (bad) atomicOr(p.status, ST_NONFINITE);
 }
