@@ -27,6 +27,7 @@
 #include <cuda_runtime.h>
 
 #include "frkc2_internal.h"
+#include "frkc2_math.cuh"
 #include "tb2d_region.cuh"
 
 namespace frkc2 {
@@ -567,23 +568,36 @@ __global__ void __launch_bounds__(RT_THREADS, 2) k_adjrev_tb2d(const AdjTbArgs a
     dk[0][3] += wgt(bS, 3, gs.w);
   }
   if constexpr (PAIRS) {
+    // dk widened on the integer pipe (frkc2_math.cuh): a hardware conversion takes an FP64-pipe slot, 64 clocks of a
+    // sub-partition, as the sum in FP64 does (1024^2, s = 100, 8 steps, forward and backward: 9457 -> 9339 us)
+    auto store = [&](auto widen) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const size_t g = size_t(y0 + 4 * ty + r) * nx + (x0 + 4 * tx);
-      float4* lo = reinterpret_cast<float4*>(a.L_out + g);
-      double2* dr = reinterpret_cast<double2*>(a.dk + g);
+      for (int r = 0; r < 4; ++r) {
+        const size_t g = size_t(y0 + 4 * ty + r) * nx + (x0 + 4 * tx);
+        float4* lo = reinterpret_cast<float4*>(a.L_out + g);
+        double2* dr = reinterpret_cast<double2*>(a.dk + g);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (!(R.outm & (1u << (4 * r + 2 * h)))) continue;
-        lo[h] = make_float4(LX[r][h].x, LY[r][h].x, LX[r][h].y, LY[r][h].y);
-        if (a.dk) {
-          double2 d = dr[h];
-          d.x += double(dk[r][2 * h]);
-          d.y += double(dk[r][2 * h + 1]);
-          dr[h] = d;
+        for (int h = 0; h < 2; ++h) {
+          if (!(R.outm & (1u << (4 * r + 2 * h)))) continue;
+          lo[h] = make_float4(LX[r][h].x, LY[r][h].x, LX[r][h].y, LY[r][h].y);
+          if (a.dk) {
+            double2 d = dr[h];
+            d.x += widen(dk[r][2 * h]);
+            d.y += widen(dk[r][2 * h + 1]);
+            dr[h] = d;
+          }
         }
       }
-    }
+    };
+    bool slow = false, ignored = false;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) (void)widen_fast(dk[r][c], slow);
+    if (__any_sync(0xffffffffu, slow))
+      store([](float v) { return widen_hw(v); });
+    else
+      store([&](float v) { return widen_fast(v, ignored); });
   } else {
 #pragma unroll
     for (int r = 0; r < 4; ++r)
