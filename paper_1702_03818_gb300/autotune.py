@@ -56,6 +56,7 @@ def candidates(prob) -> list:
     if prob.precision == F.DFLOAT:  # the float-pair state: streaming pass or register-tiled regions
         return [F.make_tuning(k=1, kernel=2)] + [F.make_tuning(k=k, kernel=3) for k in (2, 4, 6, 8, 10)]
     if prob.ndim == 2 and prob.kappa_kind != F.KAPPA_POWER:
+        c.append(F.make_tuning())  # the library's choice: FP64 whole jobs of small grids, FP32 region shapes
         c.append(F.make_tuning(k=1, kernel=2))
         if prob.precision == F.FP32:
             c += [F.make_tuning(k=k, kernel=3) for k in (2, 3, 4, 5, 6, 8, 10, 12)]
@@ -142,7 +143,7 @@ def autotune_batch(plans, probs, dt, nsteps, u, reps: int = 2):
         cands = [F.make_tuning(k=k, tile=(0, 0, g)) for k in (6, 8, 10) for g in (1, 4, 8)]
         cands += [F.make_tuning(k=1, tile=(0, r, 1)) for r in (128, 256)]
     else:  # streaming items (k = 1) by rows per tile, and the shared-memory tile pass
-        cands = [F.make_tuning(k=1, tile=(0, r, 1)) for r in (64, 128, 256)]
+        cands = [F.make_tuning(k=1, tile=(0, r, 1)) for r in (16, 32, 64, 128, 256)]
         cands += [F.make_tuning(k=k, tile=t, kernel=1) for k in (1, 2) for t in ((64, 16, 1), (32, 32, 1))]
     scratch = [t.clone() for t in u]
     times = {}
