@@ -54,27 +54,16 @@ FP32_PEAK_TOPS = 152 * 128 * 2.07e9 / 1e12
 # with 3-operation pair differences, a float increment (product + FMA) and a 10-operation
 # TwoSum update per component
 FP32_OPS_PER_CELL_STAGE = {"fp32": 16, "dfloat": 44}
-# MIXED: 4 differences in double, their 4 conversions to float, 2 conversions of f back and
-# 4 FMA updates in double, all on the FP64 pipe (ncu: 14.5 per cell-stage with the halo lane)
-MIXED_FP64_INST_PER_CELL_STAGE = 14
+# MIXED on a periodic grid: 4 differences and 4 FMA updates in double on the FP64 pipe (the
+# conversions between double and float run on the integer pipe)
+MIXED_FP64_INST_PER_CELL_STAGE = 8
 # dram bytes per launch from one ncu capture of each pass kernel, keyed by the source hash of
 # the kernel file at capture time (the value is reported only while the source is unchanged)
 NCU_TRAFFIC = {
-    # profiles/stream2d_fp64_varkappa2d_2048.md: two intermediate passes, mean of
-    # (170.4 + 42.7) MB and (170.0 + 40.1) MB
-    ("pass_stream2d.cu", "4e3d07b4b9363912"): 211.6e6,
+    # two intermediate passes at 2048^2, mean of
+    # (170.0 + 42.8) MB and (170.1 + 43.0) MB
+    ("pass_stream2d.cu", "ff9d7437f82655ef"): 212.9e6,
 }
-
-
-def wf2d_recompute(nx, ny, k=8, sms=152, ctas_per_sm=3):
-    """Computed / output cell-stages of the FP32 wavefront pass at its default launch: strips of
-    256 columns with 2h = 16 halo columns (h = k rounded up to 4), one wave of 3 CTAs per SM
-    (ncu occupancy), chunks of H rows in which every level runs H + 2k rows."""
-    h = (k + 3) // 4 * 4
-    strips = -(-nx // (256 - 2 * h))
-    chunks = max(1, min(ny, sms * ctas_per_sm // strips))
-    H = -(-ny // chunks)
-    return strips * 256 / nx * (H + 2 * k) / H
 
 
 def kernel_source_hash(name: str) -> str:
@@ -324,15 +313,14 @@ def run_ours(args, rank, world, local_rank):
             pass_bytes = cells * (npv * (4 * sbytes + kbytes) - 2 * sbytes)
             g = pass_bytes * nsteps / (smsec / 1e3) / 1e9
             if prec in FP32_OPS_PER_CELL_STAGE:
-                # k = 8 passes: compute bound (the FP32 pipe and issue).  FP32 runs the wavefront
-                # pass (strips of 256 columns, 16 halo columns; chunks of H rows, every level
-                # running H + 16 rows); DFLOAT the 64 x 64 register-tiled regions ((64/48)^2)
+                # k = 8 passes over 64 x 64 register-tiled regions ((64/48)^2 cells computed): compute
+                # bound (the FP32 pipe and issue)
                 ops = FP32_OPS_PER_CELL_STAGE[prec]
                 ach = ops * cells * s * nsteps / (smsec / 1e3) / 1e12
                 roof = {"bound": "alu", "achieved": ach, "peak": FP32_PEAK_TOPS, "unit": "Tops/s (FP32 pipe)",
                         "frac": ach / FP32_PEAK_TOPS, "ops_per_cell_stage": ops,
-                        "halo_recompute": wf2d_recompute(n, n) if prec == "fp32" else (64 / 48) ** 2,
-                        "kernel": "k_wf2d<8> (wavefront, TMA row ring)" if prec == "fp32" else "k_tb2d_df (regions)",
+                        "halo_recompute": (64 / 48) ** 2,
+                        "kernel": "k_tb2d_reg (regions)" if prec == "fp32" else "k_tb2d_df (regions)",
                         "hbm_achieved_gbs": g, "hbm_frac": g / peak_hbm, "traffic": None}
             else:  # MIXED, k = 1 streaming: bound by the FP64 pipe
                 ach = MIXED_FP64_INST_PER_CELL_STAGE * cells * s * nsteps / (smsec / 1e3) / 1e12

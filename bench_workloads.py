@@ -19,7 +19,7 @@ Workloads (sizes and seeds from frkc2_inputs.CONFIGS):
   ssweep       4096^2 var-kappa, s in {32, 128, 512, 1024}, 4 steps, FP32 vs FP64 error growth
                with s (internal amplification).
   bruss2d      the paper's Brusselator (Sec. 3.1): 200^2 periodic, s = 16, dt = 0.9 beta/rho, to
-               t = 1, FP64 and FP32, persistent launch vs one launch per stage; plus 2048^2,
+               t = 1, FP64 and FP32, the library's choice, the persistent launch, one launch per stage; plus 2048^2,
                s = 64, 10 steps for throughput against the FP64-pipe and HBM rooflines.
 """
 from __future__ import annotations
@@ -549,7 +549,7 @@ def bruss2d(F, hbm_peak_gbs: float = 6787.2):
                 dt = cfg["cfl"] * beta / rho
             v, w = v0d.clone(), w0d.clone()
             row = {"rho_bound": rho, "dt": dt, "nsteps": nsteps}
-            for kern, name in ((1, "persistent"), (2, "per_stage")):
+            for kern, name in ((0, "library_choice"), (1, "persistent"), (2, "per_stage")):
                 t = F.make_tuning(kernel=kern)
 
                 def job():
@@ -566,7 +566,7 @@ def bruss2d(F, hbm_peak_gbs: float = 6787.2):
                     tinst = cs * BRUSS_INST_PER_CELL_STAGE / (med / 1e3) / 1e12
                     r["roofline"] = {"bound": "alu", "achieved": tinst, "peak": FP64_PEAK_TINST,
                                      "unit": "Tinst/s (FP64 pipe)", "frac": tinst / FP64_PEAK_TINST}
-                else:
+                elif kern:  # (the library's FP32 passes keep k stages in registers)
                     gbs = cs * BRUSS_BYTES_PER_CELL_STAGE[prec] / (med / 1e3) / 1e9
                     r["roofline"] = {"bound": "hbm", "achieved": gbs, "peak": hbm_peak_gbs, "unit": "GB/s",
                                      "frac": gbs / hbm_peak_gbs,

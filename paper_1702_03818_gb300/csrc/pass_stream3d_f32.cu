@@ -10,7 +10,7 @@
 // The plane loop is unrolled by three with the roles of the three planes held rotated (no register
 // moves), and the passes between a step's first and last are instantiated for interleaved state.
 // 256^3, kappa(u), s = 32: 125 -> 79 us a pass (40 us at the copy bandwidth; 90 instructions a computed
-// cell against 239 an output cell before, at 62 % issue).
+// cell against 239 an output cell before, at 66 % issue).
 #include <algorithm>
 
 #include <cuda_runtime.h>
