@@ -558,7 +558,7 @@ frkc2_status frkc2_bruss_step(frkc2_plan_t plan, const frkc2_bruss_problem* prob
     if (bruss_resident_wins(*prob, plan->s, nsteps, L.total - L.flags)) {
       const cudaError_t re = launch_bruss_resident(*prob, *plan, dt, nsteps, static_cast<double*>(v), static_cast<double*>(w),
                                                    wsb + L.flags, L.total - L.flags, reinterpret_cast<unsigned*>(wsb + L.status),
-                                                   wait_limit, fault, st);
+                                                   tune ? tune->wait_limit : 0, fault, st);
       return re == cudaSuccess ? FRKC2_OK : FRKC2_ECUDA;
     }
   }

@@ -288,7 +288,7 @@ cudaError_t launch_bruss_resident(const frkc2_bruss_problem& p, const frkc2_plan
   a->nsteps = nsteps;
   a->s = plan.s;
   a->fault_inject = fault_inject;
-  a->wait_limit = wait_limit;
+  a->wait_limit = wait_limit > 0 ? wait_limit : RESIDENT_WAIT;
   a->Dd = p.D / (p.dx * p.dx);
   a->A = p.A;
   a->B1 = p.B + 1.0;

@@ -284,7 +284,7 @@ cudaError_t launch_resident2d(const frkc2_problem& p, const frkc2_plan_s& plan, 
   a->nsteps = nsteps;
   a->s = plan.s;
   a->fault_inject = fault_inject;
-  a->wait_limit = wait_limit > 0 ? wait_limit : 1ll << 22;
+  a->wait_limit = wait_limit > 0 ? wait_limit : RESIDENT_WAIT;
   const double h2 = p.dx * p.dx;
   for (int l = 0; l < plan.s; ++l) {
     a->ca[l] = dt * plan.a_re[l] / h2;

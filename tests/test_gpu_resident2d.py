@@ -88,6 +88,38 @@ def test_two_streams():
     assert all(np.array_equal(a, b) for a, b in zip(*out))
 
 
+def test_beside_a_persistent_launch():
+    """A whole job queued while a persistent batched launch holds the SMs' registers on another stream: both end as alone."""
+    s, n = 64, 600
+    plan = F.frkc2_plan(s)
+    probs, us, dts = [], [], []
+    for i in range(6):
+        u0, field = seeded_case((n, n), "periodic", "field", 70 + i)
+        kt = torch.as_tensor(field, device="cuda")
+        probs.append(F.make_problem(2, (n, n), 1.0, "periodic", "field", "fp64", kappa_field=kt))
+        us.append(torch.as_tensor(u0, device="cuda"))
+        dts.append(0.9 * O.beta(s) / O.rho_bound(oracle_problem(2, "periodic", "field", 1.0, field)))
+    steps, plans = [4] * 6, [plan] * 6
+    u0, pr, ws, opr, rho = setup(512, 500, "periodic")
+    dt, side = 0.9 * O.beta(s) / rho, torch.cuda.Stream()
+    out = []
+    for together in (False, True):
+        bu, u = [t.clone() for t in us], torch.as_tensor(u0, device="cuda").clone()
+        bws = torch.empty(F.frkc2_batch_workspace_size(plans, probs, steps), dtype=torch.uint8, device="cuda")
+        F.frkc2_workspace_reset(bws)
+        F.frkc2_batch_prepare(plans, probs, dts, steps, bu, bws)
+        torch.cuda.synchronize()
+        F.frkc2_batch_launch(bws)
+        if not together:
+            torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            F.frkc2_step(plan, pr, dt, 3, 0.0, u, ws)
+        torch.cuda.synchronize()
+        assert F.frkc2_workspace_status(ws) == F.OK and F.frkc2_workspace_status(bws) == F.OK
+        out.append([t.cpu().numpy() for t in bu + [u]])
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
+
+
 def test_status():
     s = 8
     u0, pr, ws, opr, rho = setup(60, 50, "dirichlet")
