@@ -414,8 +414,8 @@ frkc2_status frkc2_bruss_rho_bound(const frkc2_bruss_problem* prob, const void* 
 /* Advances (v, w) by nsteps FRKC2 steps of size dt (in place; v and w distinct device arrays
  * of the problem's precision).  rho > 0: dt*rho <= beta is checked (FRKC2_EUNSTABLE).
  * tune->kernel: 0 = library choice (FP32: passes of up to 8 stages in registers, the same
- * results; FP64: up to about 550^2 and 1024 stages the whole job in one cooperative launch with
- * the state in registers, its waits and fault_inject as in 1; else as 1); 1 = one persistent cooperative launch for every stage of every step,
+ * results; FP64 with up to 1024 stages: the whole job in one cooperative launch with the state in
+ * registers where that is modelled faster, its waits and fault_inject as in 1; else as 1); 1 = one persistent cooperative launch for every stage of every step,
  * each CTA waiting between stages for the CTAs whose cells its stencil reads (per-CTA stage
  * flags), or for FP64 stages of more than 2048 cells a CTA at a device-wide barrier (a plan of
  * more than 1024 stages takes one launch per 1024 stages of each step); 2 = one launch per

@@ -8,7 +8,7 @@
 // Re v^2 and Re v^2 w, the other the imaginary parts).  That is 21 FP64 instructions a row of 16 cells against 20.5,
 // in pieces that spread over the sub-partitions; a cell's operations are those of k_bruss2d (results 2e-14 apart: the
 // compiler contracts other products there).  The reaction terms, which need no neighbour, are formed while the edges
-// travel.  us a stage, persistent kernel / here: 64^2 4.2 / 2.0, 200^2 5.8 / 4.5, 300^2 9.4 / 8.0, 500^2 25.9 / 22.5;
+// travel.  us a stage, persistent kernel / here: 64^2 4.2 / 2.0, 200^2 5.8 / 4.5, 300^2 9.4 / 8.0, 388 x 535 22.3 / 18.5;
 // of the 4.5 at 200^2, 3.3 are FP64 issue, the rest the edges' trip, the barrier and the chain of a row.
 #include <algorithm>
 #include <memory>
@@ -23,7 +23,7 @@ namespace frkc2 {
 namespace {
 
 constexpr int BZ_MAXS = 1024;
-constexpr int BZ_RMAX = 8;
+constexpr int BZ_RMAX = 7;  // (8 rows a warp spill, and no grid is faster with them than in the persistent kernel)
 constexpr int bz_wmax(int R) { return R <= 2 ? 24 : 16; }  // warps (units) of a CTA
 
 struct BrussResidentArgs {
@@ -257,12 +257,20 @@ cudaError_t launch_r(const BrussResidentArgs& a, cudaStream_t st) {
 
 }  // namespace
 
-// wherever a shape fits, up to about 550^2
+// Where the model's time, with 3 % for its error (8 % for 7 rows, whose registers spill), is below what the
+// persistent kernel takes at least, the lower edge of 60 grids measured with both: 2.8 us + 0.0625 per 1000 cells, at
+// least 4.2, and steps with its CTAs a SM above that (resident / persistent us: 64 x 53 3.4 / 4.4, 183 x 176 3.8 / 5.2,
+// 395 x 238 8.7 / 9.6, 255 x 720 16.3 / 19.2; on the other side 420 x 269 11.3 / 10.4, 147 x 1816 26.3 / 22.6: strips and
+// bands of uneven units).
 bool bruss_resident_wins(const frkc2_bruss_problem& p, int s, int nsteps, size_t packet_bytes) {
   if (p.precision != FRKC2_FP64 || s > BZ_MAXS || (long long)nsteps * s >= 0x7fffffffll) return false;
   if (p.nx * p.ny > (1 << 20)) return false;
   const CoopDevice d = coop_device();
-  return d.coop && bruss_resident_shape(int(p.nx), int(p.ny), d.sms, packet_bytes).R > 0;
+  if (!d.coop) return false;
+  const BrussResidentShape sh = bruss_resident_shape(int(p.nx), int(p.ny), d.sms, packet_bytes);
+  const double cells = double(p.nx) * double(p.ny), per_sm = cells / (256.0 * d.sms);
+  const double persistent = per_sm > 6.0 ? 22.4 : per_sm > 4.0 ? 19.0 : std::max(4.2, 2.8 + 0.0625e-3 * cells);
+  return sh.R > 0 && sh.us * (sh.R >= 7 ? 1.08 : 1.03) <= persistent;
 }
 
 cudaError_t launch_bruss_resident(const frkc2_bruss_problem& p, const frkc2_plan_s& plan, double dt, int nsteps, double* v, double* w,
@@ -304,8 +312,7 @@ cudaError_t launch_bruss_resident(const frkc2_bruss_problem& p, const frkc2_plan
     case 4: return launch_r<4>(*a, st);
     case 5: return launch_r<5>(*a, st);
     case 6: return launch_r<6>(*a, st);
-    case 7: return launch_r<7>(*a, st);
-    default: return launch_r<8>(*a, st);
+    default: return launch_r<7>(*a, st);
   }
 }
 
