@@ -1,0 +1,33 @@
+"""Which kernels a call launches, and with which grids, without a GPU: the library's host code over a stand-in runtime
+that checks launches against the limits of the real one (fake_runtime.py)."""
+import math
+
+import pytest
+
+import fake_runtime as R
+
+
+@pytest.fixture(scope="module")
+def F(tmp_path_factory):
+    return R.load(str(tmp_path_factory.mktemp("fake")))
+
+
+def bruss(F, nx, ny, prec, s=16, nsteps=1, bc="periodic", tune=None):
+    p = F.make_bruss_problem((nx, ny), bc=bc, precision=prec)
+    ws = R.Buffer(F.frkc2_bruss_workspace_size(p), 1 << 41)
+    F._lib.fake_reset()
+    F.frkc2_bruss_step(F.frkc2_plan(s), p, 1e-4, nsteps, 0.0, R.Buffer(1), R.Buffer(1, 1 << 42), ws, tune, stream=0)
+    return R.launches(F)
+
+
+@pytest.mark.parametrize("bc", ["periodic", "neumann"])
+@pytest.mark.parametrize("nx,ny", [(16, 2_000_000), (1, 1 << 24), (256, 4_000_000), (4_000_000, 256), (200, 200)])
+def test_bruss_fp32_takes_tall_grids(F, nx, ny, bc):
+    """Every pass has a CTA for each of its regions, however many rows of them there are."""
+    got = bruss(F, nx, ny, "fp32", bc=bc)
+    assert {g.kernel for g in got} == {"k_bruss_tb2d"}
+    cells = {16 * (2 if "Li2E" in g.mangled else 4) for g in got}
+    assert len(cells) == 1
+    edge = cells.pop()
+    for g in got:
+        assert any(math.prod(g.grid) == -(-nx // (edge - 2 * k)) * -(-ny // (edge - 2 * k)) for k in range(1, 9))
