@@ -406,6 +406,9 @@ static TbShape tb2d_best(int C, int nx, int ny, int s, int kmin, int kstep, int 
   for (int k = kmin; k <= std::min(s, kmax); k += kstep) {
     auto pass = [&](int q) {
       const int T = 16 * C - 2 * q;
+      // A launch's y axis ends at 65535: tall grids take regions high enough, up to 4 million rows.  (Regions along one
+      // axis would have no such end, but the registers of their division cost a 2048^2 pass 6 %: 3931 -> 4176 us, s = 64, 10 steps.)
+      if ((ny + T - 1) / T > 65535) return 1e30;
       return tb2d_pass_us(C, q, (long long)((nx + T - 1) / T) * ((ny + T - 1) / T), sms);
     };
     const double us = (s / k) * pass(k) + (s % k ? pass(s % k) : 0.0);

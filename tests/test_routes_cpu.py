@@ -31,3 +31,24 @@ def test_bruss_fp32_takes_tall_grids(F, nx, ny, bc):
     edge = cells.pop()
     for g in got:
         assert any(math.prod(g.grid) == -(-nx // (edge - 2 * k)) * -(-ny // (edge - 2 * k)) for k in range(1, 9))
+
+
+def step(F, n, prec, bc="periodic", kappa="const", s=16, nsteps=1, tune=None):
+    p = F.make_problem(len(n), n, 1.0, bc, kappa, prec)
+    if kappa == "field":
+        p.kappa = 1 << 43
+    ws = R.Buffer(F.frkc2_workspace_size(p), 1 << 41)
+    F._lib.fake_reset()
+    F.frkc2_step(F.frkc2_plan(s), p, 1e-4, nsteps, 0.0, R.Buffer(1), ws, tune, stream=0)
+    return R.launches(F)
+
+
+@pytest.mark.parametrize("bc", ["periodic", "dirichlet"])
+@pytest.mark.parametrize("nx,ny", [(12, 2_000_000), (16, 1_500_000), (24, 1_400_000), (1, 3_000_000), (301, 3_900_000), (100, 100)])
+def test_fp32_2d_takes_tall_grids(F, nx, ny, bc):
+    """Every pass has a CTA for each of its regions, however many rows of them there are."""
+    got = [g for g in step(F, (nx, ny), "fp32", bc, s=32) if g.kernel != "k_faces_padded"]
+    assert {g.kernel for g in got} == {"k_tb2d_reg"}
+    edge = 16 * (2 if "Li2E" in got[0].mangled else 4)
+    for g in got:
+        assert any(math.prod(g.grid) == -(-nx // (edge - 2 * k)) * -(-ny // (edge - 2 * k)) for k in range(1, 13))
