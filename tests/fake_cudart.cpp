@@ -106,7 +106,7 @@ cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {
 }
 // (as if every kernel took 64 registers a thread, those of 4 x 4 cells a thread 128)
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void* f, int threads, size_t smem, unsigned) {
-  const int regs = names()[f].find("tb2d") != std::string::npos && names()[f].find("Li2E") == std::string::npos ? 128 : 64;
+  const int regs = names()[f].find("tb2d") != std::string::npos && names()[f].find("ILi2E") == std::string::npos ? 128 : 64;
   *n = 65536 / (regs * threads);
   if (smem) *n = std::min(*n, int(size_t(228 * 1024) / (smem + 1024)));
   return cudaSuccess;

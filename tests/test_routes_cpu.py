@@ -26,7 +26,7 @@ def test_bruss_fp32_takes_tall_grids(F, nx, ny, bc):
     """Every pass has a CTA for each of its regions, however many rows of them there are."""
     got = bruss(F, nx, ny, "fp32", bc=bc)
     assert {g.kernel for g in got} == {"k_bruss_tb2d"}
-    cells = {16 * (2 if "Li2E" in g.mangled else 4) for g in got}
+    cells = {16 * (2 if "ILi2E" in g.mangled else 4) for g in got}
     assert len(cells) == 1
     edge = cells.pop()
     for g in got:
@@ -49,6 +49,6 @@ def test_fp32_2d_takes_tall_grids(F, nx, ny, bc):
     """Every pass has a CTA for each of its regions, however many rows of them there are."""
     got = [g for g in step(F, (nx, ny), "fp32", bc, s=32) if g.kernel != "k_faces_padded"]
     assert {g.kernel for g in got} == {"k_tb2d_reg"}
-    edge = 16 * (2 if "Li2E" in got[0].mangled else 4)
+    edge = 16 * (2 if "ILi2E" in got[0].mangled else 4)
     for g in got:
         assert any(math.prod(g.grid) == -(-nx // (edge - 2 * k)) * -(-ny // (edge - 2 * k)) for k in range(1, 13))
