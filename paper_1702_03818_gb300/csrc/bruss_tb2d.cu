@@ -39,7 +39,6 @@ struct BrTbArgs {
   const float* in[4];   // Re v, Im v, Re w, Im w; the imaginary parts nullptr: zero
   float* out[4];        // the imaginary parts nullptr: not stored
   int nx, ny, k;
-  int cols;             // regions across
   float Dd, A, B1, B;   // D / dx^2, A, B + 1, B
   int check_finite;
   int vec;              // rows of C cells are aligned and never wrap: whole-row loads and stores
@@ -142,7 +141,7 @@ __global__ void __launch_bounds__(BT_THREADS, C == 4 ? 2 : 4) k_bruss_tb2d(const
   BrTbShared<C>& sh = *reinterpret_cast<BrTbShared<C>*>(smem_raw);
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int k = p.k, T = BT_R - 2 * k, nx = p.nx, ny = p.ny;
-  const int rx = int(blockIdx.x) % p.cols * T - k, ry = int(blockIdx.x) / p.cols * T - k;  // the region's corner
+  const int rx = blockIdx.x * T - k, ry = blockIdx.y * T - k;  // the region's corner
   const int x0 = rx + C * tx, y0 = ry + C * ty;
   // launched with programmatic stream serialization: the next pass may start its CTAs as this one's
   // exit, and every global load below comes after the previous launch has completed
@@ -216,14 +215,13 @@ Residency bt_residency() {
 }
 
 template <int C, bool PERIODIC>
-cudaError_t bt_launch(BrTbArgs a, cudaStream_t st, bool overlap_previous) {
+cudaError_t bt_launch(const BrTbArgs& a, cudaStream_t st, bool overlap_previous) {
   const Residency res = bt_residency<C, PERIODIC>();
   if (res.err != cudaSuccess) return res.err;
   const int T = 16 * C - 2 * a.k;
-  a.cols = (a.nx + T - 1) / T;
-  const long long regions = (long long)a.cols * ((a.ny + T - 1) / T);
+  const long long regions = (long long)((a.nx + T - 1) / T) * ((a.ny + T - 1) / T);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned(regions), 1, 1);  // (along one axis: a grid's y ends at 65535, 1.6 million rows of cells here)
+  cfg.gridDim = dim3((a.nx + T - 1) / T, (a.ny + T - 1) / T, 1);
   cfg.blockDim = dim3(BT_THREADS, 1, 1);
   cfg.dynamicSmemBytes = spread_smem(sizeof(BrTbShared<C>), regions, res.sms, res.per_sm);
   cfg.stream = st;
@@ -267,6 +265,10 @@ BrussTb bruss_tb2d_shape(int nx, int ny, int s) {
       }
     }
   }
+  // A launch's y axis ends at 65535: where the regions of a pass are more (from 1.5 million rows on), the persistent
+  // kernel.  (Regions along one axis would have no such end, but 2048^2, s = 16, 10 steps, takes 2213 -> 2250 us with them.)
+  for (int k : {best.k, best.k ? s % best.k : 0})
+    if (k > 0 && (ny - 1) / (16 * best.cells - 2 * k) >= 65535) return BrussTb{0, 0};
   return best;
 }
 

@@ -8,9 +8,10 @@ F = pytest.importorskip("paper_1702_03818_gb300.frkc2")
 
 
 @pytest.mark.parametrize("bc", ["periodic", "neumann"])
-def test_bruss_fp32(bc):
+@pytest.mark.parametrize("nx,ny", [(16, 2_000_000), (16, 1_400_000)])
+def test_bruss_fp32(nx, ny, bc):
     """The same bits as one launch a stage, which has no regions."""
-    nx, ny, s = 16, 2_000_000, 16
+    s = 16
     pr = F.make_bruss_problem((nx, ny), dx=1.0 / 200, bc=bc, precision="fp32")
     plan = F.frkc2_plan(s)
     g = torch.Generator(device="cuda").manual_seed(5)
