@@ -698,6 +698,7 @@ int adj_tb2d_k(const frkc2_problem& p, int s, bool rev) {
   }();
   auto pass = [&](int k) {
     const dim3 g = region_grid(p, k);
+    if (g.y > 65535) return 1e30;  // (the end of a launch's y axis)
     const long long regions = (long long)g.x * g.y, slots = 2ll * sms, full = regions / slots, rest = regions % slots;
     auto wave = [&](long long ctas) {
       if (rev) return ctas > sms ? 22.0 + 2.45 * k : 13.0 + 1.75 * k;

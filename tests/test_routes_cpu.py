@@ -50,3 +50,22 @@ def test_fp32_2d_takes_tall_grids(F, nx, ny, bc):
     edge = 16 * (2 if "ILi2E" in got[0].mangled else 4)
     for g in got:
         assert any(math.prod(g.grid) == -(-nx // (edge - 2 * k)) * -(-ny // (edge - 2 * k)) for k in range(1, 13))
+
+
+def adjoint(F, n, prec, s, nsteps, ckpt, bc="periodic"):
+    p = F.make_problem(len(n), n, 1.0, bc, "field", prec)
+    p.kappa = 1 << 50
+    plan = F.frkc2_plan(s)
+    ws = R.Buffer(F.frkc2_adjoint_workspace_size(plan, p, nsteps, ckpt), 1 << 41)
+    F._lib.fake_reset()
+    F.frkc2_adjoint(plan, p, 1e-4, nsteps, ckpt, *(R.Buffer(1, (42 + i) << 40) for i in range(4)), ws, stream=0)
+    return R.launches(F)
+
+
+@pytest.mark.parametrize("nx,ny", [(8, 2_900_000), (2, 3_000_000), (100, 3_100_000), (100, 100)])
+def test_fp32_adjoint_takes_tall_grids(F, nx, ny):
+    got = adjoint(F, (nx, ny), "fp32", 20, 2, 1)
+    tb = [g for g in got if g.kernel in ("k_tape_tb2d", "k_adjrev_tb2d")]
+    assert {g.kernel for g in tb} == {"k_tape_tb2d", "k_adjrev_tb2d"}
+    for g in tb:
+        assert any(math.prod(g.grid) == -(-nx // (64 - 2 * k)) * -(-ny // (64 - 2 * k)) for k in range(1, 13))
