@@ -216,7 +216,8 @@ __global__ void __launch_bounds__(AS_THREADS, adj_min_blocks<S>())
 template <class S, class A, bool PERIODIC>
 cudaError_t launch_t(const AdjStreamArgs& a, cudaStream_t st) {
   const auto kern = k_adj_stream2d<S, A, PERIODIC>;
-  static const Residency res = spread_residency(kern, AS_THREADS, 0, 0);
+  static SpreadKernel own;
+  const Residency res = spread_residency(own, kern, AS_THREADS, 0, 0);
   if (res.err != cudaSuccess) return res.err;
   const int ncolw = (a.nx + AS_COLS - 1) / AS_COLS;
   const long long total = (long long)ncolw * a.ny;

@@ -621,7 +621,8 @@ size_t adj_spread(size_t need, dim3 grid, const Residency& res) {
 template <bool PERIODIC, bool PAIRS>
 cudaError_t launch_rev(const AdjTbArgs& a, dim3 grid, cudaStream_t st) {
   const auto kern = k_adjrev_tb2d<PERIODIC, PAIRS>;
-  static const Residency res = spread_residency(kern, RT_THREADS, sizeof(RevShared), 0);
+  static SpreadKernel own;
+  const Residency res = spread_residency(own, kern, RT_THREADS, sizeof(RevShared), 0);
   if (res.err != cudaSuccess) return res.err;
   {
     cudaLaunchConfig_t cfg = {};
@@ -645,7 +646,8 @@ template <bool PERIODIC, bool PAIRS>
 cudaError_t launch_tape(const AdjTbArgs& a, dim3 grid, cudaStream_t st) {
   const auto kern = k_tape_tb2d<PERIODIC, PAIRS>;
   constexpr size_t fixed = 2 * 2 * 2 * 256 * sizeof(float4);  // its static shared memory
-  static const Residency res = spread_residency(kern, RT_THREADS, 0, fixed);
+  static SpreadKernel own;
+  const Residency res = spread_residency(own, kern, RT_THREADS, 0, fixed);
   if (res.err != cudaSuccess) return res.err;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;

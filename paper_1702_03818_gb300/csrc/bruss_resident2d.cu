@@ -245,8 +245,8 @@ BrussResidentShape bruss_resident_shape(int nx, int ny, int sms, size_t bytes) {
 template <int R>
 cudaError_t launch_r(const BrussResidentArgs& a, cudaStream_t st) {
   constexpr size_t per_warp = 2 * 4 * 2 * 32 * sizeof(double);
-  static const cudaError_t attr = cudaFuncSetAttribute((const void*)k_bruss_resident<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       int(per_warp * bz_wmax(R)));
+  static SmemLimit smem;
+  const cudaError_t attr = smem.raise(k_bruss_resident<R>, per_warp * bz_wmax(R));
   if (attr != cudaSuccess) return attr;
   void* args[] = {const_cast<BrussResidentArgs*>(&a)};
   const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_bruss_resident<R>, dim3(a.nstrip * a.nband),

@@ -210,8 +210,8 @@ __global__ void __launch_bounds__(BT_THREADS, C == 4 ? 2 : 4) k_bruss_tb2d(const
 
 template <int C, bool PERIODIC>
 Residency bt_residency() {
-  static const Residency res = spread_residency(k_bruss_tb2d<C, PERIODIC>, BT_THREADS, sizeof(BrTbShared<C>), 0);
-  return res;
+  static SpreadKernel own;
+  return spread_residency(own, k_bruss_tb2d<C, PERIODIC>, BT_THREADS, sizeof(BrTbShared<C>), 0);
 }
 
 template <int C, bool PERIODIC>

@@ -2,8 +2,10 @@
 #pragma once
 
 #include <algorithm>
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
+#include <mutex>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -269,11 +271,36 @@ inline SpreadGrid spread_grid(long long work, int sms, int per_sm) {
   const long long r = std::max<long long>(1, std::min<long long>(per_sm, (work + sms - 1) / sms));
   return {unsigned(r * sms), spread_smem(0, r * sms, sms, per_sm)};
 }
-// query_residency for a kernel launched with such padding: `fixed` bytes of static shared memory
+// A kernel's MaxDynamicSharedMemorySize belongs to the device that is current when it is set: one of these per kernel
+// sets it once on each device that launches the kernel (from the 65th on at every launch).
+class SmemLimit {
+  std::atomic<unsigned long long> done_{0};
+
+ public:
+  template <class K>
+  cudaError_t raise(K kern, size_t bytes) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (done_.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+    if (e == cudaSuccess) done_.fetch_or(bit, std::memory_order_relaxed);
+    return e;
+  }
+};
+
+// query_residency for a kernel launched with such padding: `fixed` bytes of static shared memory.  `own`: the kernel's.
+struct SpreadKernel {
+  SmemLimit smem;
+  std::once_flag once;
+  Residency res{cudaSuccess, 0, 0};
+};
 template <class K>
-Residency spread_residency(K kern, int threads, size_t smem, size_t fixed) {
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SPREAD_SMEM - fixed));
-  Residency r = query_residency(kern, threads, smem);
+Residency spread_residency(SpreadKernel& own, K kern, int threads, size_t smem, size_t fixed) {
+  const cudaError_t e = own.smem.raise(kern, SPREAD_SMEM - fixed);
+  std::call_once(own.once, [&] { own.res = query_residency(kern, threads, smem); });
+  Residency r = own.res;
   if (e != cudaSuccess) r.err = e;
   return r;
 }

@@ -161,7 +161,8 @@ __global__ void __launch_bounds__(PR_THREADS, FRKC2_PAIRED_MIN_BLOCKS)
 template <class S, class A, bool PERIODIC>
 cudaError_t launch_t(const PassArgs& a, const void* fen, cudaStream_t st) {
   const auto kern = k_paired2d<S, A, PERIODIC>;
-  static const Residency res = spread_residency(kern, PR_THREADS, 0, 0);
+  static SpreadKernel own;
+  const Residency res = spread_residency(own, kern, PR_THREADS, 0, 0);
   if (res.err != cudaSuccess) return res.err;
   const int ncolw = (a.nx + PR_COLS - 1) / PR_COLS;
   const long long total = (long long)ncolw * a.ny;

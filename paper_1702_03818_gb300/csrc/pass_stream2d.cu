@@ -293,7 +293,8 @@ __global__ void k_face_pairs(const A* __restrict__ fx, const A* __restrict__ fy,
 template <class S, class A, bool PERIODIC, bool HAT>
 cudaError_t launch_t(const PassArgs& a, const void* fen, cudaStream_t st) {
   const auto kern = k_stream2d<S, A, PERIODIC, HAT>;
-  static const Residency res = spread_residency(kern, ST_THREADS, 0, 0);
+  static SpreadKernel own;
+  const Residency res = spread_residency(own, kern, ST_THREADS, 0, 0);
   if (res.err != cudaSuccess) return res.err;
   const int ncolw = (a.nx + ST_COLS - 1) / ST_COLS;
   const long long total = (long long)ncolw * a.ny;  // (chunk, row) pairs

@@ -223,7 +223,8 @@ __global__ void __launch_bounds__(DF_THREADS, DF_MIN_BLOCKS)
 template <bool PERIODIC, bool IN_REAL, bool OUT_REAL>
 cudaError_t launch_t(const PassArgs& a, const void* fen, cudaStream_t st) {
   const auto kern = k_stream2d_df<PERIODIC, IN_REAL, OUT_REAL>;
-  static const Residency res = spread_residency(kern, DF_THREADS, 0, 0);
+  static SpreadKernel own;
+  const Residency res = spread_residency(own, kern, DF_THREADS, 0, 0);
   if (res.err != cudaSuccess) return res.err;
   const int ncolw = (a.nx + DF_COLS - 1) / DF_COLS;
   const long long total = (long long)ncolw * a.ny;

@@ -348,9 +348,8 @@ __global__ void __launch_bounds__(RT_THREADS, C == 4 ? 2 : 4) k_tb2d_reg(const P
 
 template <int C, bool PERIODIC, int VEC>
 Residency tb_residency() {
-  static const Residency res =
-      spread_residency(k_tb2d_reg<C, PERIODIC, VEC>, RT_THREADS, 0, sizeof(typename Row<C>::type) * 2 * 2 * 2 * 256);
-  return res;
+  static SpreadKernel own;
+  return spread_residency(own, k_tb2d_reg<C, PERIODIC, VEC>, RT_THREADS, 0, sizeof(typename Row<C>::type) * 2 * 2 * 2 * 256);
 }
 
 template <int C, bool PERIODIC, int VEC>

@@ -50,7 +50,8 @@ __global__ void __launch_bounds__(RT_THREADS, 2) k_tb2d_df(const PassArgs p, con
 template <bool PERIODIC, bool IN_REAL, bool OUT_REAL>
 cudaError_t launch_t(const PassArgs& a, const DfIo& io, cudaStream_t st, bool overlap_previous) {
   const auto kern = k_tb2d_df<PERIODIC, IN_REAL, OUT_REAL>;
-  static const Residency res = spread_residency(kern, RT_THREADS, sizeof(DfShared), 0);
+  static SpreadKernel own;
+  const Residency res = spread_residency(own, kern, RT_THREADS, sizeof(DfShared), 0);
   if (res.err != cudaSuccess) return res.err;
   const int T = RT_R - 2 * a.k;
   cudaLaunchConfig_t cfg = {};

@@ -62,7 +62,7 @@ const char* fake_launch(int i) {
 }
 void fake_reset() {
   log_.clear();
-  refuse_coop = device = 0;
+  refuse_coop = 0;
   last = cudaSuccess;
 }
 void fake_refuse_cooperative(int error) { refuse_coop = error; }

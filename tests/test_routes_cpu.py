@@ -69,3 +69,29 @@ def test_fp32_adjoint_takes_tall_grids(F, nx, ny):
     assert {g.kernel for g in tb} == {"k_tape_tb2d", "k_adjrev_tb2d"}
     for g in tb:
         assert any(math.prod(g.grid) == -(-nx // (64 - 2 * k)) * -(-ny // (64 - 2 * k)) for k in range(1, 13))
+
+
+def test_second_device(F):
+    """Calls on a second GPU of the process launch what they launch on the first (a kernel's shared memory limit is set on
+    each device)."""
+    def runs():
+        out = []
+        for prec in ("fp64", "fp32", "mixed", "dfloat"):
+            for n in ((100, 90), (700, 611)):
+                out.append(lambda n=n, prec=prec: step(F, n, prec, kappa="field"))
+                out.append(lambda n=n, prec=prec: step(F, n, prec, "dirichlet", tune=F.make_tuning(k=1)))
+        for prec in ("fp64", "fp32"):
+            out += [lambda prec=prec: bruss(F, 120, 90, prec), lambda prec=prec: adjoint(F, (120, 90), prec, 16, 2, 1)]
+        p = F.make_problem(2, (90, 80), 1.0, "periodic", "const", "fp64")
+        ws, plan = R.Buffer(F.frkc2_workspace_size(p), 1 << 41), F.frkc2_plan(16, flags=F.PLAN_PAIRED)
+        out.append(lambda: (F._lib.fake_reset(), F.frkc2_step(plan, p, 1e-4, 1, 0.0, R.Buffer(1), ws, stream=0), R.launches(F))[2])
+        return out
+
+    for run in runs():
+        first = run()
+        try:
+            F._lib.cudaSetDevice(1)
+            second = run()
+        finally:
+            F._lib.cudaSetDevice(0)
+        assert [g._replace(device=1) for g in first] == second and {g.device for g in second} == {1}
