@@ -469,8 +469,9 @@ bool segment_resident(const AdjCtx& C, int m) {
 }
 bool run_segment_resident(const AdjCtx& C, int j, int m) {
   if (cudaMemcpyAsync(C.ckpt(j + 1), C.ckpt(j), C.N * C.SB, cudaMemcpyDeviceToDevice, C.st) != cudaSuccess) return false;
-  return launch_resident2d(*C.p, *C.plan, C.dt, m, C.ckpt(j + 1), C.base + C.L.fx, C.base + C.L.fy, C.base + C.L.tape,
-                           C.L.lam - C.L.tape, reinterpret_cast<unsigned*>(C.base + C.L.status), 0, 0, C.st) == cudaSuccess;
+  const cudaError_t e = launch_resident2d(*C.p, *C.plan, C.dt, m, C.ckpt(j + 1), C.base + C.L.fx, C.base + C.L.fy, C.base + C.L.tape,
+                                          C.L.lam - C.L.tape, reinterpret_cast<unsigned*>(C.base + C.L.status), 0, 0, C.st);
+  return coop_refused(e) ? run_segment(C, j) : e == cudaSuccess;
 }
 
 frkc2_status adj_forward(const AdjCtx& C, const void* u0) {

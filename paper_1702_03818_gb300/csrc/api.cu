@@ -311,7 +311,7 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
   if (use_stream2d && kern == 0 && !(tune && tune->k) && resident2d_wins(p, s, nsteps, L.total - L.fen)) {
     const cudaError_t e = launch_resident2d(p, *plan, dt, nsteps, u, base + L.fx, base + L.fy, base + L.fen, L.total - L.fen,
                                             a.status, tune ? tune->wait_limit : 0, tune ? tune->fault_inject : 0, st);
-    return e == cudaSuccess ? FRKC2_OK : FRKC2_ECUDA;
+    if (!coop_refused(e)) return e == cudaSuccess ? FRKC2_OK : FRKC2_ECUDA;
   }
   const void* curU = u;
   const void* curV = nullptr;

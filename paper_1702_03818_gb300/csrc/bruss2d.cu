@@ -559,7 +559,7 @@ frkc2_status frkc2_bruss_step(frkc2_plan_t plan, const frkc2_bruss_problem* prob
       const cudaError_t re = launch_bruss_resident(*prob, *plan, dt, nsteps, static_cast<double*>(v), static_cast<double*>(w),
                                                    wsb + L.flags, L.total - L.flags, reinterpret_cast<unsigned*>(wsb + L.status),
                                                    tune ? tune->wait_limit : 0, fault, st);
-      return re == cudaSuccess ? FRKC2_OK : FRKC2_ECUDA;
+      if (!coop_refused(re)) return re == cudaSuccess ? FRKC2_OK : FRKC2_ECUDA;
     }
   }
   const bool per = prob->bc == FRKC2_BC_PERIODIC;

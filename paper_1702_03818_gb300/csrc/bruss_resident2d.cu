@@ -251,7 +251,7 @@ cudaError_t launch_r(const BrussResidentArgs& a, cudaStream_t st) {
   void* args[] = {const_cast<BrussResidentArgs*>(&a)};
   const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_bruss_resident<R>, dim3(a.nstrip * a.nband),
                                                     dim3(32 * a.cw * a.rh), args, per_warp * a.cw * a.rh, st);
-  count_launch();
+  if (e == cudaSuccess) count_launch();
   return e;
 }
 

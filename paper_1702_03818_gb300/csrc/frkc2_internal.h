@@ -158,7 +158,14 @@ bool resident2d_wins(const frkc2_problem& p, int s, int nsteps, size_t packet_by
 cudaError_t launch_resident2d(const frkc2_problem& p, const frkc2_plan_s& plan, double dt, int nsteps, void* u, const void* fx,
                               const void* fy, void* packets, size_t packet_bytes, unsigned* status, long long wait_limit,
                               int fault_inject, cudaStream_t st);
-// the same for the Brusselator in FP64 (bruss_resident2d.cu)
+// A cooperative launch that the context cannot hold at once (it may have fewer SMs than the device): nothing has run,
+// and the caller takes the form of a launch a stage.
+inline bool coop_refused(cudaError_t e) {
+  const bool refused = e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported || e == cudaErrorLaunchOutOfResources;
+  if (refused) (void)cudaGetLastError();
+  return refused;
+}
+// the same for the Brusselator in FP64 (bruss_resident2d.cu; refused: the persistent kernel)
 bool bruss_resident_wins(const frkc2_bruss_problem& p, int s, int nsteps, size_t packet_bytes);
 cudaError_t launch_bruss_resident(const frkc2_bruss_problem& p, const frkc2_plan_s& plan, double dt, int nsteps, double* v, double* w,
                                   void* packets, size_t packet_bytes, unsigned* status, long long wait_limit, int fault_inject,

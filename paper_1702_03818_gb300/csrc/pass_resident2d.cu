@@ -242,7 +242,7 @@ cudaError_t launch_r(const Resident2dArgs& a, cudaStream_t st) {
   void* args[] = {const_cast<Resident2dArgs*>(&a)};
   const cudaError_t e =
       cudaLaunchCooperativeKernel((const void*)k_resident2d<R>, dim3(a.nstrip * a.nband), dim3(32 * a.cw * a.rh), args, 0, st);
-  count_launch();
+  if (e == cudaSuccess) count_launch();
   return e;
 }
 

@@ -62,7 +62,6 @@ const char* fake_launch(int i) {
 }
 void fake_reset() {
   log_.clear();
-  refuse_coop = 0;
   last = cudaSuccess;
 }
 void fake_refuse_cooperative(int error) { refuse_coop = error; }

@@ -95,3 +95,25 @@ def test_second_device(F):
         finally:
             F._lib.cudaSetDevice(0)
         assert [g._replace(device=1) for g in first] == second and {g.device for g in second} == {1}
+
+
+@pytest.mark.parametrize("error", [720, 801, 701])  # too large for a cooperative launch, not supported, out of resources
+def test_refused_cooperative_launch(F, error):
+    """Where the context refuses the whole job in one launch, a call takes the launch per stage (the Brusselator, whose
+    other form is cooperative too, still says so)."""
+    def kernels(run):
+        return {g.kernel for g in run()}
+
+    calls = [lambda: step(F, (100, 90), "fp64", kappa="field"), lambda: adjoint(F, (100, 90), "fp64", 16, 4, 1)]
+    plain = [kernels(c) for c in calls]
+    assert all("k_resident2d" in k for k in plain)
+    F._lib.fake_refuse_cooperative(error)
+    try:
+        assert kernels(calls[0]) == {"k_faces", "k_face_pairs", "k_stream2d"}
+        assert kernels(calls[1]) == plain[1] - {"k_resident2d"}
+        with pytest.raises(F.Frkc2Error):
+            bruss(F, 100, 90, "fp64")
+        assert len(bruss(F, 100, 90, "fp64", tune=F.make_tuning(kernel=2))) == 16
+    finally:
+        F._lib.fake_refuse_cooperative(0)
+    assert [kernels(c) for c in calls] == plain
