@@ -628,7 +628,7 @@ cudaError_t launch_rev(const AdjTbArgs& a, dim3 grid, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(RT_THREADS, 1, 1);
-        cfg.dynamicSmemBytes = adj_spread(sizeof(RevShared), grid, res);
+    cfg.dynamicSmemBytes = adj_spread(sizeof(RevShared), grid, res);
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -689,7 +689,10 @@ dim3 region_grid(const frkc2_problem& p, int k) {
 // Stages of a tape (rev = false) or reverse pass: 8, or for pair access the even count whose passes take the
 // least by a model of their time in us fitted to measurements (k = 4 .. 12, periodic grids of 100^2 to 1500^2): a
 // wave with one or two regions an SM, waves overlapping by c at their ends.  Model / measured: reverse 1024^2
-// k = 8 79 / 78, k = 10 89 / 93; tape 1024^2 k = 8 35 / 32, k = 10 39 / 38, 300 x 277 k = 12 15.8 / 16.2.
+// k = 8 79 / 78; tape 1024^2 k = 8 35 / 32, k = 10 39 / 38, 300 x 277 k = 12 15.8 / 16.2.  A reverse pass has at most
+// 8 stages: it sums dJ/dkappa over them in FP32, and the sums of the passes in FP64.  (Forward and backward in us, most
+// 12 / most 8: 100^2, s = 32, 4 steps 464 / 504, 640^2, s = 64, 2 steps 761 / 780, 1024^2, s = 100, 8 steps 9270 / 9003;
+// 12 with the first 8 added to the FP64 sum inside the pass 491, 778, 9493.)
 int adj_tb2d_k(const frkc2_problem& p, int s, bool rev) {
   if (!adj_pairs(p, 8)) return 8;
   static const int sms = [] {
@@ -711,7 +714,7 @@ int adj_tb2d_k(const frkc2_problem& p, int s, bool rev) {
   };
   int best = 8;
   double least = 0.0;
-  for (int k = 4; k <= 12; k += 2) {
+  for (int k = 4; k <= (rev ? 8 : 12); k += 2) {
     const double us = (s / k) * pass(k) + (s % k ? pass(s % k) : 0.0);
     if (k == 4 || us < least) {
       best = k;
