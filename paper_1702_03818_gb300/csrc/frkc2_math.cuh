@@ -81,7 +81,10 @@ __device__ __forceinline__ void kappa_power(T u, T v, T c, T p, T& kr, T& ki) {
     }
   }
   kr = T(1) + c * wr;
-  ki = c * wi;
+  if constexpr (std::is_same<T, double>::value)
+    ki = __dmul_rn(c, wi);  // (not for the caller to fuse with a sum, as below)
+  else
+    ki = c * wi;
 }
 
 // ---- double <-> float on the integer pipe ------------------------------------------------------
@@ -183,10 +186,12 @@ __device__ __forceinline__ void kappa_power25_fast(T x, T y, T c, T& kr, T& ki) 
   const T sr = x >= T(0) ? t : h;
   const T si = copysign(x >= T(0) ? h : t, y);
   const T qr = fma(x, x, -yy), qi = (x + x) * y;
-  const T wr = qr * sr - qi * si, wi = qr * si + qi * sr;
+  // (Which products are fused is written out, and ki is not for the caller to fuse with a sum: the same bits wherever
+  // this is inlined.  An unrolled plane loop fused it in every other plane.)
+  const T wr = fma(qr, sr, -mul_rn(qi, si)), wi = fma(qr, si, mul_rn(qi, sr));
   const T cs = c * T(0.70710678118654752440);  // loop-invariant
   kr = fma(cs, wr, T(1));
-  ki = cs * wi;
+  ki = mul_rn(cs, wi);
 }
 
 }  // namespace frkc2

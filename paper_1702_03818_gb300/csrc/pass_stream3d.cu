@@ -8,7 +8,7 @@
 //   - each cell forms the fluxes through its east, north and up faces, F = kappa_f (W_nb - W_c); the
 //     west flux is lane - 1's east flux (shuffle), the down flux the up flux of the plane below
 //     (register), and inside a thread's rows the south flux is the north flux of the row below:
-//     f = (F_e - F_w) + (F_n - F_s) + (F_u - F_d), every face flux formed once;
+//     f = (F_e - F_w) + (F_n - F_s) + (F_u - F_d), every face flux formed once (MIXED: see flux);
 //   - between warps, the y exchange runs one plane ahead: a warp publishes its first row's W and
 //     kappa of plane z + 1 and its last row's north flux of plane z (formed during plane z - 1) in
 //     the same double-buffered shared write, so one barrier a plane serves both directions;
@@ -136,9 +136,11 @@ __global__ void __launch_bounds__(32 * S3_MAXW) k_stream3d(const S3Args p) {
     if (POWER) k.y = a.y + b.y;
     return k;
   };
-  // (Which product of the imaginary part is fused is fixed here, so that a MIXED call's bits do not
-  // depend on the compiler's choice: the x and y faces one way, the z faces the other, and the down
-  // faces of every 32nd plane as the x and y faces -- the bits of a pass over 32-plane chunks.)
+  // (Which product of the imaginary part is fused is fixed here, so that results depend neither on the
+  // compiler's choice nor on where the chunks along z begin: the x and y faces one way, the z faces the
+  // other.  MIXED only: plane 32 j takes its down face as the x and y faces, so that this one face of 32 has
+  // two fluxes, a float rounding apart.  These are the results that MIXED has had since its chunks were of 32
+  // planes; with one flux there the state moves by 5e-9 in norm, 121 x 150 x 97, 32 stages, more than double results may.)
   auto flux = [&](A2 kf, A dr, A di, bool zface) -> A2 {
     A2 F;
     if (POWER) {
@@ -242,7 +244,7 @@ __global__ void __launch_bounds__(32 * S3_MAXW) k_stream3d(const S3Args p) {
           Kc[r] = loadk(zc, r);
           Kp[r] = loadk(zp, r);
         }
-        Fd[r] = face(Wc[r], Wm, Kc[r], Km, z0 % S3_CHUNK != 0);
+        Fd[r] = face(Wc[r], Wm, Kc[r], Km, !MIX || z0 % S3_CHUNK != 0);
       }
       shW[b][w][lane] = Wc[0];
       shK[b][w][lane] = Kc[0];
