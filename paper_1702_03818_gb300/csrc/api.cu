@@ -256,7 +256,6 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
       use_stream2d = stream_ok;
     }
   }
-  if (use_stream3d) use_stream3d = stream3d_supported(p);  // (else the tile pass)
   if (use_stream2d && !(tune && tune->tile_y)) ty = 64;
   {
     PassArgs probe{};

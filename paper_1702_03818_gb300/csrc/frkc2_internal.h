@@ -171,7 +171,6 @@ cudaError_t launch_bruss_resident(const frkc2_bruss_problem& p, const frkc2_plan
                                   void* packets, size_t packet_bytes, unsigned* status, long long wait_limit, int fault_inject,
                                   cudaStream_t st);
 int stream3d_chunks(long long blocks, int nz, long long slots);
-bool stream3d_supported(const frkc2_problem& p);
 cudaError_t launch_pass_stream3d_f32(const frkc2_problem& p, const PassArgs& a, cudaStream_t st);
 cudaError_t launch_pass_stream3d(const frkc2_problem& p, const PassArgs& a, cudaStream_t st);
 // faces in padded rows (a.fx, a.fy of pitch fpitch), the pair state between passes as four planes of `plane` floats in

@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(32 * S3_MAXW) k_stream3d(const S3Args p) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int lane = threadIdx.x, w = threadIdx.y, nw = blockDim.y;
   const int nx = p.nx, ny = p.ny, nz = p.nz;
-  const size_t plane = size_t(nx) * ny;  // at most 2^32 (stream3d_supported)
+  const size_t plane = size_t(nx) * ny;
   const bool in_real = p.in_real, out_real = p.out_real;
   const S ca = S(p.ca), cb = S(p.cb);
   const A kc = A(p.kc), kp = A(p.kp);
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(32 * S3_MAXW) k_stream3d(const S3Args p) {
     // per row: the in-plane offset read (wrapped, or clamped to the grid: the conductivity of a
     // Dirichlet ghost is its interior cell's), whether the row is in the grid / an output row, and
     // whether a neighbour needs it
-    unsigned col[RY];
+    size_t col[RY];
     unsigned inside = 0, act = 0, need = 0;  // bits by row; act and need are warp-uniform
     const bool xin = PERIODIC || (gx >= 0 && gx < nx);
     const int xr = PERIODIC ? wrap3(gx, nx) : min(max(gx, 0), nx - 1);
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(32 * S3_MAXW) k_stream3d(const S3Args p) {
     for (int r = 0; r < RY; ++r) {
       const int gy = gy0 + r, R = w * RY + r;
       const int yr = PERIODIC ? wrap3(gy, ny) : min(max(gy, 0), ny - 1);
-      col[r] = unsigned(yr) * unsigned(nx) + unsigned(xr);
+      col[r] = size_t(yr) * nx + xr;
       if (xin && (PERIODIC || (gy >= 0 && gy < ny))) inside |= 1u << r;
       if (R >= 1 && R <= p.oy && gy < ny) act |= 1u << r;
       if (gy <= ny) need |= 1u << r;
@@ -427,11 +427,6 @@ int stream3d_chunks(long long blocks, int nz, long long slots) {
   return best;
 }
 
-// In-plane offsets are 32-bit, in FP32 in bytes (a larger plane takes the tile pass).
-bool stream3d_supported(const frkc2_problem& p) {
-  return p.ndim == 3 && p.n[0] * p.n[1] <= (int64_t(1) << (p.precision == FRKC2_FP32 ? 29 : 32));
-}
-
 cudaError_t launch_pass_stream3d(const frkc2_problem& p, const PassArgs& a, cudaStream_t st) {
   S3Args s{};
   s.nx = a.nx;
@@ -450,7 +445,8 @@ cudaError_t launch_pass_stream3d(const frkc2_problem& p, const PassArgs& a, cuda
   s.status = a.status;
   switch (p.precision) {
     case FRKC2_FP64: return launch_s<double, double>(p, s, st);
-    case FRKC2_FP32: return launch_pass_stream3d_f32(p, a, st);
+    case FRKC2_FP32:  // (its offsets in a plane are 32-bit, in bytes)
+      return p.n[0] * p.n[1] <= (int64_t(1) << 29) ? launch_pass_stream3d_f32(p, a, st) : launch_s<float, float>(p, s, st);
     default: return launch_s<double, float>(p, s, st);
   }
 }

@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(32 * F3_MAXW, F3_CTAS) k_stream3d_f32(const F3
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int lane = threadIdx.x, w = threadIdx.y, nw = blockDim.y;
   const int nx = p.nx, ny = p.ny, nz = p.nz;
-  const size_t plane = size_t(nx) * ny;  // at most 2^29 (stream3d_supported): offsets in a plane are 32-bit
+  const size_t plane = size_t(nx) * ny;  // at most 2^29 (launch_pass_stream3d): offsets in a plane are 32-bit
   const bool in_real = !CC && p.in_real, out_real = !CC && p.out_real;
   const float2 ca2 = make_float2(p.ca, p.ca), cb2 = make_float2(p.cb, p.cb), ncb2 = make_float2(-p.cb, -p.cb);
   const float kc = p.kc, cs = p.kc * 0.70710678118654752440f;

@@ -117,3 +117,11 @@ def test_refused_cooperative_launch(F, error):
     finally:
         F._lib.fake_refuse_cooperative(0)
     assert [kernels(c) for c in calls] == plain
+
+
+@pytest.mark.parametrize("prec,n,kernel", [("fp32", (2048, 300_000, 1), "k_stream3d"), ("fp32", (2048, 200_000, 2), "k_stream3d_f32"),
+                                           ("fp32", (70_000, 70_000, 1), "k_stream3d"), ("fp64", (70_000, 70_000, 1), "k_stream3d"),
+                                           ("mixed", (16_000, 300_000, 1), "k_stream3d")])
+def test_3d_streams_planes_of_any_size(F, prec, n, kernel):
+    got = step(F, n, prec, kappa="power", s=4)
+    assert [g.kernel for g in got] == [kernel] * 4
