@@ -411,18 +411,22 @@ cudaError_t launch_s(const frkc2_problem& p, const S3Args& a, cudaStream_t st) {
 
 }  // namespace
 
-// Chunks along z: the count whose waves of CTAs (slots resident at once) take the fewest planes, two
-// more per chunk for its priming.  Column blocks of one chunk are neighbours in the launch order, so
-// the CTAs that run together read the same planes and share their halo columns and lines in L2.
+// Chunks along z: of 1 .. min(nz, 256), the count whose waves of CTAs (slots resident at once) take the fewest planes,
+// two more per chunk for its priming, the smallest of equal ones.  Column blocks of one chunk are neighbours in the launch
+// order, so the CTAs that run together read the same planes and share their halo columns and lines in L2.
+// Every stage's launch asks, so it looks only at the smallest count with the chunk length of the most chunks that w waves
+// hold, until w waves take more planes however long their chunks are (nz = 250: 1.2 us of the host for a look at every count).
 int stream3d_chunks(long long blocks, int nz, long long slots) {
+  const int most = std::min(nz, 256);
   int best = 1;
-  long long least = 0;
-  for (int c = 1; c <= std::min(nz, 256); ++c) {
-    const long long planes = (blocks * c + slots - 1) / slots * ((nz + c - 1) / c + 2);
-    if (c == 1 || planes < least) {
-      best = c;
-      least = planes;
+  long long least = (blocks + slots - 1) / slots * (nz + 2);  // one chunk
+  for (long long w = (blocks + slots - 1) / slots; blocks * nz + 2 * w * slots < least * slots; ++w) {
+    const long long c = std::min<long long>(most, w * slots / blocks), length = (nz + c - 1) / c;
+    if (w * (length + 2) < least) {
+      best = int((nz + length - 1) / length);
+      least = w * (length + 2);
     }
+    if (c == most) break;
   }
   return best;
 }

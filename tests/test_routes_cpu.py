@@ -1,6 +1,9 @@
 """Which kernels a call launches, and with which grids, without a GPU: the library's host code over a stand-in runtime
 that checks launches against the limits of the real one (fake_runtime.py)."""
+import ctypes
 import math
+import random
+import time
 
 import pytest
 
@@ -125,3 +128,35 @@ def test_refused_cooperative_launch(F, error):
 def test_3d_streams_planes_of_any_size(F, prec, n, kernel):
     got = step(F, n, prec, kappa="power", s=4)
     assert [g.kernel for g in got] == [kernel] * 4
+
+
+def chunks(F):
+    f = F._lib._ZN5frkc215stream3d_chunksExix
+    f.argtypes, f.restype = [ctypes.c_longlong, ctypes.c_int, ctypes.c_longlong], ctypes.c_int
+    return f
+
+
+def test_3d_chunks_are_the_best_of_all_counts(F):
+    """The number of chunks along z is that of a look at every count: fewest planes over its waves, then fewest chunks."""
+    f, r = chunks(F), random.Random(3)
+    for _ in range(3000):
+        nz, slots = int(math.exp(r.uniform(0, 7))), 152 * r.randint(1, 8)
+        blocks = int(math.exp(r.uniform(0, 9)))
+        planes = [(-(-blocks * c // slots) * (-(-nz // c) + 2), c) for c in range(1, min(nz, 256) + 1)]
+        assert f(blocks, nz, slots) == min(planes)[1], (blocks, nz, slots)
+
+
+def test_3d_chunks_cost_a_launch_little(F):
+    """Every stage asks: a tall box takes about the time of a flat one, most of it the call from here."""
+    f = chunks(F)
+
+    def us(nz):
+        best = math.inf
+        for _ in range(30):
+            t = time.perf_counter()
+            for _ in range(500):
+                f(3, nz, 608)
+            best = min(best, (time.perf_counter() - t) / 500 * 1e6)
+        return best
+
+    assert us(250) < 2 * us(1)
