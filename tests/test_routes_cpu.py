@@ -160,3 +160,31 @@ def test_3d_chunks_cost_a_launch_little(F):
         return best
 
     assert us(250) < 2 * us(1)
+
+
+# The sizes at which the GPU tests compare these kernels with others, and some on the other side of each rule.
+@pytest.mark.parametrize("s", [6, 16, 1024])
+@pytest.mark.parametrize("nx,ny", [(1, 1), (1, 9), (9, 1), (16, 4), (15, 16), (33, 21), (64, 64), (7, 300), (300, 7), (200, 200), (256, 256),
+                                   (400, 400), (34, 411), (457, 355), (247, 777), (619, 305)])
+def test_bruss_fp64_small_grids_in_registers(F, nx, ny, s):
+    got = bruss(F, nx, ny, "fp64", s=s, nsteps=2)
+    assert [(g.kernel, g.cooperative) for g in got] == [("k_bruss_resident", True)]
+    assert got[0].grid[0] <= 152
+
+
+@pytest.mark.parametrize("nx,ny,s", [(500, 512, 16), (610, 600, 16), (420, 269, 16), (2048, 2048, 16), (64, 64, 1026)])
+def test_bruss_fp64_larger_grids_persistent(F, nx, ny, s):
+    assert {g.kernel for g in bruss(F, nx, ny, "fp64", s=s)} == {"k_bruss2d"}
+
+
+@pytest.mark.parametrize("nx,ny,s,passes", [(2, 3, 4, 2), (24, 20, 16, 2), (96, 33, 10, 2), (144, 144, 16, 2), (700, 611, 12, 3),
+                                            (2048, 1030, 16, 2)])
+def test_bruss_fp32_stages_in_few_passes(F, nx, ny, s, passes):
+    assert [g.kernel for g in bruss(F, nx, ny, "fp32", s=s)] == ["k_bruss_tb2d"] * passes
+
+
+@pytest.mark.parametrize("nx,ny,s,nsteps,ckpt,plain", [(5, 8, 6, 4, 1, 3), (33, 21, 16, 5, 2, 2), (97, 130, 32, 4, 1, 3), (200, 200, 16, 7, 3, 2),
+                                                       (700, 700, 16, 2, 1, 0), (33, 21, 16, 5, 5, 0)])
+def test_fp64_adjoint_forward_segments_in_one_launch(F, nx, ny, s, nsteps, ckpt, plain):
+    """Every segment but the last runs forward in one launch where the grid fits."""
+    assert [g.kernel for g in adjoint(F, (nx, ny), "fp64", s, nsteps, ckpt)].count("k_resident2d") == plain
