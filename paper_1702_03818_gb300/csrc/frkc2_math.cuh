@@ -171,7 +171,8 @@ __device__ __forceinline__ double rsqrt_h3(double a) {
 __device__ __forceinline__ float sqrt_h3(float a) { return a * rsqrt_n(a); }
 __device__ __forceinline__ float rsqrt_h3(float a) { return rsqrt_n(a); }
 
-// |w|^2 kept normal (below, w^2.5 vanishes against 1 whatever its square root); NaN passes through
+// |w|^2 kept normal (below, w^2.5 vanishes against 1 whatever its square root).  A NaN may come
+// back as that or as itself; it reaches kappa(w) through x or y.
 __device__ __forceinline__ double keep_normal(double m) {
   return __double2hiint(m) < 0x00100000 ? __hiloint2double(0x00100000, 0) : m;
 }
@@ -192,6 +193,30 @@ __device__ __forceinline__ void kappa_power25_fast(T x, T y, T c, T& kr, T& ki) 
   const T cs = c * T(0.70710678118654752440);  // loop-invariant
   kr = fma(cs, wr, T(1));
   ki = mul_rn(cs, wi);
+}
+
+// two floats to an instruction (sm_100 family)
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+// kappa(w) = 1 + c w^2.5 of a pair; cs = c / sqrt(2)
+__device__ __forceinline__ void kappa25_pair(float2 x, float2 y, float cs, float2& kr, float2& ki) {
+  const float2 yy = mul2(y, y), m = fma2(x, x, yy);
+  const float2 mc = make_float2(keep_normal(m.x), keep_normal(m.y));
+  const float2 r = mul2(mc, make_float2(rsqrt_n(mc.x), rsqrt_n(mc.y)));
+  const float2 b = make_float2(r.x + fabsf(x.x), r.y + fabsf(x.y));
+  const float2 q = make_float2(rsqrt_n(b.x), rsqrt_n(b.y));
+  const float2 t = mul2(b, q), h = make_float2(fabsf(y.x) * q.x, fabsf(y.y) * q.y);
+  const bool p0 = x.x >= 0.f, p1 = x.y >= 0.f;
+  const float2 sr = make_float2(p0 ? t.x : h.x, p1 ? t.y : h.y);
+  const float2 si = make_float2(copysignf(p0 ? h.x : t.x, y.x), copysignf(p1 ? h.y : t.y, y.y));
+  const float2 qr = fma2(make_float2(-2.f, -2.f), yy, m), nqr = mul2(make_float2(-1.f, -1.f), qr);
+  const float2 nqi = mul2(mul2(make_float2(-2.f, -2.f), x), y);
+  const float2 wr = fma2(nqi, si, mul2(qr, sr));
+  const float2 nwi = fma2(nqi, sr, mul2(nqr, si));
+  kr = fma2(make_float2(cs, cs), wr, make_float2(1.f, 1.f));
+  ki = mul2(make_float2(-cs, -cs), nwi);
 }
 
 }  // namespace frkc2
