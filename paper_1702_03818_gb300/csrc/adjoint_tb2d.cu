@@ -695,12 +695,7 @@ dim3 region_grid(const frkc2_problem& p, int k) {
 // 12 with the first 8 added to the FP64 sum inside the pass 491, 778, 9493.)
 int adj_tb2d_k(const frkc2_problem& p, int s, bool rev) {
   if (!adj_pairs(p, 8)) return 8;
-  static const int sms = [] {
-    int dev = 0, n = 152;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      n = 152;
-    return n;
-  }();
+  const int sms = model_sms();
   auto pass = [&](int k) {
     const dim3 g = region_grid(p, k);
     if (g.y > 65535) return 1e30;  // (the end of a launch's y axis)

@@ -714,17 +714,6 @@ struct BatchPlanHost {
   long long total_items;
 };
 
-// SMs of the device (152 where it cannot be asked).
-int batch_sms() {
-  static const int sms = [] {
-    int dev = 0, n = 152;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      n = 152;
-    return n;
-  }();
-  return sms;
-}
-
 // FP32 and DFLOAT region items: consecutive 64 x 64 regions of one pass per work item (tune->tile_z), which
 // spreads the per-item hand-over (ticket, decode, dependency check, completion fence) over several regions.  The
 // default is up to 4, fewer where a round has too few regions to go round: one per item below 3 regions a
@@ -734,7 +723,7 @@ int batch_sms() {
 int batch_group(int precision, const frkc2_tuning* tune, bool streaming, double regions_per_round) {
   if (streaming || (precision != FRKC2_FP32 && precision != FRKC2_DFLOAT)) return 1;
   if (tune && tune->tile_z) return tune->tile_z;
-  return std::max(1, std::min(4, int(regions_per_round / (1.5 * 2 * batch_sms()))));
+  return std::max(1, std::min(4, int(regions_per_round / (1.5 * 2 * model_sms()))));
 }
 
 // FP64 / MIXED batches with one stage per pass run streaming items unless kernel 1 (the shared-
@@ -764,7 +753,7 @@ int batch_stream_rows(int nprob, const frkc2_plan_t* plans, const frkc2_problem*
     rows += double((probs[i].n[0] + BS_COLS - 1) / BS_COLS) * double(probs[i].n[1]) * passes;
     most = std::max(most, passes);
   }
-  const double r = rows / most / (1.15 * 2 * batch_sms());
+  const double r = rows / most / (1.15 * 2 * model_sms());
   return r >= 128.0 ? 128 : std::max(8, int(r / 8.0) * 8);
 }
 

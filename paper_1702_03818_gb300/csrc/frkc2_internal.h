@@ -253,6 +253,17 @@ Residency query_residency(K kern, int threads, size_t smem) {
   return r;
 }
 
+// SMs for the models of a pass's time: the device's, or 152 where it cannot be asked.
+inline int model_sms() {
+  static const int sms = [] {
+    int dev = 0, n = 152;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      n = 152;
+    return n;
+  }();
+  return sms;
+}
+
 // Dynamic shared memory that spreads a launch of `ctas` CTAs over the SMs: where they fit in one wave, as
 // much as leaves room for just ceil(ctas / sms) of them per SM.  CTAs of a dependent launch that starts
 // early (programmatic stream serialization) are otherwise packed onto the SMs that empty first: a pass of

@@ -1,4 +1,5 @@
-// Device helpers: principal-branch complex power for kappa(w) = 1 + c w^p.
+// Device helpers: periodic index, principal-branch complex power for kappa(w) = 1 + c w^p, conversions between
+// double and float.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -6,6 +7,13 @@
 #include <type_traits>
 
 namespace frkc2 {
+
+// A cell index on a periodic axis (g >= -n).
+__device__ __forceinline__ int wrap3(int g, int n) {
+  if (g < 0) g += n;
+  while (g >= n) g -= n;
+  return g;
+}
 
 // Principal square root of x + i y (branch cut on the negative real axis; the sign of a
 // zero imaginary part selects the side, as in C99 csqrt), from the half-angle formulas
@@ -47,16 +55,6 @@ __device__ __forceinline__ void csqrt_principal(T x, T y, T& rr, T& ri) {
     rr = h;
     ri = copysign(t, y);
   }
-}
-
-// kappa(w) = 1 + c w^2.5 = 1 + c w^2 sqrt(w) for complex w = u + i v (principal branch).
-template <class T>
-__device__ __forceinline__ void kappa_power25(T u, T v, T c, T& kr, T& ki) {
-  T sr, si;
-  csqrt_principal<T>(u, v, sr, si);  // sqrt(0) = 0, so 0^2.5 = 0 needs no test
-  const T qr = u * u - v * v, qi = T(2) * u * v;
-  kr = T(1) + c * (qr * sr - qi * si);
-  ki = c * (qr * si + qi * sr);
 }
 
 // kappa(w) = 1 + c w^p for complex w = u + i v on the principal branch, 0^p = 0 (p > 0).
@@ -127,6 +125,7 @@ __device__ __forceinline__ double widen_hw(float f) {
   return r;
 }
 
+// products that the compiler never fuses into a neighbouring add
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 

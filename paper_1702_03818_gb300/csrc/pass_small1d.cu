@@ -27,6 +27,7 @@
 #include <cuda_runtime.h>
 
 #include "frkc2_internal.h"
+#include "frkc2_math.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -53,11 +54,6 @@ struct Small1dArgs {
   double ca[S1_MAXS];    // dt Re a_l / dx^2
   double cb[S1_MAXS];    // dt Im a_l / dx^2
 };
-
-// products that are never contracted into a neighbouring add: every cell position of every
-// launch shape then rounds the same way, so all shapes give the same bits
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 
 __device__ __forceinline__ bool bad1(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
 __device__ __forceinline__ bool bad1(float v) { return (__float_as_uint(v) & 0x7f800000u) == 0x7f800000u; }

@@ -56,12 +56,6 @@ template <> struct V2s<float> { using type = float2; };
 
 __device__ __forceinline__ bool nonfinite3(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
 
-__device__ __forceinline__ int wrap3(int g, int n) {
-  if (g < 0) g += n;
-  while (g >= n) g -= n;
-  return g;
-}
-
 // Rows of one thread and the most warps of a CTA.  160^3, kappa(u), a pass: 16 warps FP64 668 us /
 // MIXED 139 us; FP64 with 12 warps 669 us, 8 warps (2 CTAs per SM) 703 us, 4 warps (4 CTAs) 771 us:
 // with the FP64 pipe the bound, the halo rows of smaller CTAs cost more than they hide.

@@ -52,12 +52,6 @@ struct F3Args {
   unsigned* status;
 };
 
-__device__ __forceinline__ int wrapf3(int g, int n) {
-  if (g < 0) g += n;
-  while (g >= n) g -= n;
-  return g;
-}
-
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(make_float2(-1.f, -1.f), b, a); }  // exact product
 
 // One plane of a thread's rows: two pairs of complex states and conductivities.
@@ -130,11 +124,11 @@ __global__ void __launch_bounds__(32 * F3_MAXW, F3_CTAS) k_stream3d_f32(const F3
     // the grid, of `outm`: it is an output
     unsigned off[RY], inside = 0, outm = 0;
     const bool xin = PERIODIC || (gx >= 0 && gx < nx);
-    const int xr = PERIODIC ? wrapf3(gx, nx) : min(max(gx, 0), nx - 1);
+    const int xr = PERIODIC ? wrap3(gx, nx) : min(max(gx, 0), nx - 1);
 #pragma unroll
     for (int r = 0; r < RY; ++r) {
       const int gy = gy0 + r, R = w * RY + r;
-      const int yr = PERIODIC ? wrapf3(gy, ny) : min(max(gy, 0), ny - 1);
+      const int yr = PERIODIC ? wrap3(gy, ny) : min(max(gy, 0), ny - 1);
       off[r] = (unsigned(yr) * unsigned(nx) + unsigned(xr)) * 8u;
       if (xin && (PERIODIC || (gy >= 0 && gy < ny))) inside |= 1u << r;
       if (out_x && R >= 1 && R <= p.oy && gy < ny) outm |= 1u << r;
@@ -144,11 +138,11 @@ __global__ void __launch_bounds__(32 * F3_MAXW, F3_CTAS) k_stream3d_f32(const F3
     unsigned poff;
     {
       const int gy = gy0 + (lane >> 3), px = gx - lane + 4 * (lane & 7);
-      poff = (unsigned(PERIODIC ? wrapf3(gy, ny) : min(max(gy, 0), ny - 1)) * unsigned(nx) +
-              unsigned(PERIODIC ? wrapf3(px, nx) : min(max(px, 0), nx - 1))) * 8u;
+      poff = (unsigned(PERIODIC ? wrap3(gy, ny) : min(max(gy, 0), ny - 1)) * unsigned(nx) +
+              unsigned(PERIODIC ? wrap3(px, nx) : min(max(px, 0), nx - 1))) * 8u;
     }
     auto prefetch = [&](int z) {
-      const char* base = static_cast<const char*>(p.in) + size_t(PERIODIC ? wrapf3(z, nz) : min(max(z, 0), nz - 1)) * plane * 8;
+      const char* base = static_cast<const char*>(p.in) + size_t(PERIODIC ? wrap3(z, nz) : min(max(z, 0), nz - 1)) * plane * 8;
       if (in_bounds(poff / 8 < plane, p.status)) {
         asm volatile("prefetch.global.L2 [%0];" ::"l"(base + poff));
         if (!POWER && p.kappa && (lane & 1) == 0)
@@ -158,7 +152,7 @@ __global__ void __launch_bounds__(32 * F3_MAXW, F3_CTAS) k_stream3d_f32(const F3
     };
     // W (and FIELD / CONST conductivities) of plane z; the offsets are 32-bit against a uniform base
     auto load = [&](int z, Plane3& q) {
-      const size_t zo = size_t(PERIODIC ? wrapf3(z, nz) : min(max(z, 0), nz - 1)) * plane;
+      const size_t zo = size_t(PERIODIC ? wrap3(z, nz) : min(max(z, 0), nz - 1)) * plane;
       const char* base = static_cast<const char*>(p.in) + zo * (in_real ? 4 : 8);
       const char* kbase = reinterpret_cast<const char*>(p.kappa) + zo * 4;
 #pragma unroll

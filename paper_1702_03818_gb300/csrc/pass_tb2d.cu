@@ -395,12 +395,7 @@ static double tb2d_pass_us(int C, int k, long long regions, int sms) {
 }
 
 static TbShape tb2d_best(int C, int nx, int ny, int s, int kmin, int kstep, int kmax) {
-  static const int sms = [] {
-    int dev = 0, n = 152;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      n = 152;
-    return n;
-  }();
+  const int sms = model_sms();
   TbShape best{C, kmin, 0.0};
   for (int k = kmin; k <= std::min(s, kmax); k += kstep) {
     auto pass = [&](int q) {

@@ -482,12 +482,7 @@ double wf2d_pass8_us(int nx, int ny) { return 8.8e-6 * double(nx) * ny * wf2d_re
 double wf2d_recompute(int nx, int ny, int k) {
   // strips of 256 columns with 2h halo columns; one wave of 3 CTAs per SM (the occupancy of the
   // k <= 8 instantiations); chunks of H rows in which every level runs H + 2k rows
-  static const int sms = [] {
-    int dev = 0, n = 152;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      n = 152;
-    return n;
-  }();
+  const int sms = model_sms();
   const int h = (k + 3) / 4 * 4, ow = 64 * WF_NW - 2 * h;
   const int strips = (nx + ow - 1) / ow;
   const int chunks = std::max(1, std::min(ny, 3 * sms / strips));
