@@ -117,7 +117,7 @@ typedef struct {
                         pass of 1, 2, 4, 6, 8, 10 or 12 stages; the FP32 2D default there)  */
   long long wait_limit; /* batched launch, FP64 2D whole job and kernel 7 (its waits on the TMA row copies):
                         polls a device wait makes before it gives up and latches
-                        FRKC2_ETIMEOUT (0 = library default: 2^22 polls, whole jobs 2^25)   */
+                        FRKC2_ETIMEOUT (0 = library default: 2^22 polls, whole jobs 2^28)   */
   int fault_inject;  /* testing only: 1 = in the batched launch the first dependent work
                         item waits on a counter nothing advances; in the FP64 2D whole job
                         the first wait is for a stage nothing publishes; in kernel 7 (passes of
@@ -419,7 +419,7 @@ frkc2_status frkc2_bruss_rho_bound(const frkc2_bruss_problem* prob, const void* 
  * each CTA waiting between stages for the CTAs whose cells its stencil reads (per-CTA stage
  * flags), or for FP64 stages of more than 2048 cells a CTA at a device-wide barrier (a plan of
  * more than 1024 stages takes one launch per 1024 stages of each step); 2 = one launch per
- * stage.  The waits are bounded by tune->wait_limit polls (0 = 2^22, whole jobs in registers 2^25); on expiry FRKC2_ETIMEOUT
+ * stage.  The waits are bounded by tune->wait_limit polls (0 = 2^22, whole jobs in registers 2^28); on expiry FRKC2_ETIMEOUT
  * is latched in the workspace and the launch returns early (the state is then unspecified).
  * tune->fault_inject = 1 (testing only, persistent form) makes the first wait between stages
  * wait for a count that nothing reaches.  A non-finite value in a step's output latches FRKC2_ENONFINITE.

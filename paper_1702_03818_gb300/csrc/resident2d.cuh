@@ -33,9 +33,10 @@ __device__ __forceinline__ double flip(double v, bool negate) {
   return __hiloint2double(__double2hiint(v) ^ (negate ? int(0x80000000u) : 0), __double2loint(v));
 }
 
-// Polls of a wait by default: some 20 s.  The CTAs of a launch may be placed one by one as a long launch on another
-// stream leaves the SMs, and the first of them wait for the last.
-constexpr long long RESIDENT_WAIT = 1ll << 25;
+// Polls of a wait by default: 62 s (233 ns a poll, 64^2) to 120 s (447 ns, 200^2 Brusselator).  The CTAs of a launch may be
+// placed one by one as a long launch on another stream leaves the SMs, and the first of them wait for the last: a batch of
+// 512 FP64 problems takes 7 s, which 2^25 polls (8 s) hardly outlast.
+constexpr long long RESIDENT_WAIT = 1ll << 28;
 
 struct CoopDevice {
   int sms, coop;
