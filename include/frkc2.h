@@ -114,7 +114,8 @@ typedef struct {
                         FP32 wavefront pass: strips of 256 columns walked up the grid with k
                         stage levels in flight, rows staged in shared memory by TMA bulk
                         copies (n[0] a multiple of 4 and >= 256, u 16-byte aligned, every
-                        pass of 1, 2, 4, 6, 8, 10 or 12 stages; the FP32 2D default there)  */
+                        pass of 1, 2, 4, 6, 8, 10 or 12 stages; the FP32 2D default above about
+                        3500^2 cells)                                                        */
   long long wait_limit; /* batched launch, FP64 2D whole job and kernel 7 (its waits on the TMA row copies):
                         polls a device wait makes before it gives up and latches
                         FRKC2_ETIMEOUT (0 = library default: 2^22 polls, whole jobs 2^28)   */

@@ -230,7 +230,7 @@ frkc2_status frkc2_step(frkc2_plan_t plan, const frkc2_problem* prob, double dt,
     use_wf = true;
   } else if (kern == 0) {
     // FP32 k-stage passes.  The library's choice is the cheaper by the two models of a step: the regions up to
-    // about 3000^2, the wavefront above (2048^2 6.28 against 7.26 us a stage, 4096^2 23.0 against 22.6).  For a
+    // about 3500^2, the wavefront above (2048^2 6.28 against 7.26 us a stage, 4096^2 23.0 against 22.6).  For a
     // given k, the wavefront where it recomputes fewer cells than the 64 x 64 regions, allowing for its 8 %
     // higher cost per computed cell-stage (2048^2, k = 8, single-cell accesses in the regions).
     const int nx = int(p.n[0]), ny = int(p.n[1]);

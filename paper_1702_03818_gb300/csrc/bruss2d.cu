@@ -553,7 +553,7 @@ frkc2_status frkc2_bruss_step(frkc2_plan_t plan, const frkc2_bruss_problem* prob
       return te == cudaSuccess ? FRKC2_OK : FRKC2_ECUDA;
     }
   }
-  if (kern == 0) {  // FP64 grids that fit the SMs' registers (200^2, s = 16, 42 steps 3900 -> 3020 us)
+  if (kern == 0) {  // FP64 grids that fit the SMs' registers (200^2, s = 16, 42 steps 3900 -> 2960 us)
     const BrLayout L = br_layout(*prob);
     if (bruss_resident_wins(*prob, plan->s, nsteps, L.total - L.flags)) {
       const cudaError_t re = launch_bruss_resident(*prob, *plan, dt, nsteps, static_cast<double*>(v), static_cast<double*>(w),

@@ -8,8 +8,8 @@
 // Re v^2 and Re v^2 w, the other the imaginary parts).  That is 21 FP64 instructions a row of 16 cells against 20.5,
 // in pieces that spread over the sub-partitions; a cell's operations are those of k_bruss2d (results 2e-14 apart: the
 // compiler contracts other products there).  The reaction terms, which need no neighbour, are formed while the edges
-// travel.  us a stage, persistent kernel / here: 64^2 4.2 / 2.0, 200^2 5.8 / 4.5, 300^2 9.4 / 8.0, 388 x 535 22.3 / 18.5;
-// of the 4.5 at 200^2, 3.3 are FP64 issue, the rest the edges' trip, the barrier and the chain of a row.
+// travel.  us a stage, persistent kernel / here: 64^2 4.2 / 2.0, 200^2 5.8 / 4.4, 300^2 9.4 / 8.0, 388 x 535 22.3 / 18.5;
+// of the 4.4 at 200^2, 3.3 are FP64 issue, the rest the edges' trip, the barrier and the chain of a row.
 #include <algorithm>
 #include <memory>
 

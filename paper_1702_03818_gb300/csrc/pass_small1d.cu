@@ -406,7 +406,7 @@ cudaError_t launch_small1d(const frkc2_problem& p, const frkc2_plan_s& plan, dou
   while (R * threads < ext) R *= 2;
   if (R > S1_RMAX) return cudaErrorInvalidValue;
   // FP64 in the library's own shape: components on separate lanes where that is the faster (us a stage, s = 32):
-  //   one cell a lane in up to 8 warps: ext 60 0.48 against 0.64, 90 0.58 / 0.65, 104 0.63 / 0.67; in 10 warps and
+  //   one cell a lane in up to 8 warps: ext 60 0.45 against 0.64, 90 0.58 / 0.65, 104 0.63 / 0.67; in 10 warps and
   //   more (ext > 140) 0.79 / 0.80 and 1.05 / 0.97: both issue about the same FP64 work per cell there;
   //   where one cell a thread doesn't hold the chunk: n = 4096 2.0 / 3.2, 6000 2.7 / 3.2 (the other form fills 512
   //   threads with 2^i cells each, most of them beyond the chunk).
