@@ -9,9 +9,10 @@
 // columns beyond its own come from the adjacent threads by 16-lane shuffles.  Every cell is updated by the
 // operations of k_bruss2d in their order, so the results are bit for bit those of the per-stage forms.
 //
-// What bounds it: FP32 issue (about 48 instructions a computed cell-stage, 41 of them arithmetic), and on
+// What bounds it: FP32 issue (57 instructions a computed cell-stage, 41 of them arithmetic, at 65 % issue), and on
 // grids of less than a wave the latency of a stage.  C = 4 (64 registers of state, 2 CTAs per SM) recomputes
-// least and serves large grids; C = 2 gives four times as many CTAs, for grids that would leave SMs idle.
+// least and serves large grids; at its 128 registers it spills (88 bytes stored and 220
+// loaded a thread, zero flux 148 and 288).  C = 2 gives four times as many CTAs, for grids that would leave SMs idle.
 // 2048^2, s = 16, 10 steps: 6165 -> 2218 us (41 % of the FP32 rate counting the halo); 200^2, 42 steps: 1859 ->
 // 450 us; 700 x 611 zero flux, 10 steps: 875 -> 436 us.
 #include <algorithm>
